@@ -48,7 +48,9 @@ enum {
   DMRG_ETIMEOUT = -6  /* a bounded device-side wait ran out                  */
 };
 
-/* FP64: every operation in FP64.  FP32: FP64 block operators, renormalization and
+/* FP64: every operation in FP64 accuracy (the triple products of H.psi, renormalization and
+ * density matrices as block-scaled 58-bit integers where the values allow it, no less exact
+ * than FP64 arithmetic, with FP64 sums over the tasks).  FP32: FP64 block operators, renormalization and
  * density matrices; FP32 copies of the operators for the Davidson matvecs (FP32
  * CUDA-core arithmetic).  BF16X3: FP64 block operators, renormalization and
  * density matrices; H.psi output blocks with both sides <= 128 and one side >=
@@ -144,7 +146,7 @@ int dmrg_hpsi(dmrg_ctx *ctx, const double *psi, double *sigma, int device_ptrs);
  * The first call on a device looks up that array's device address (a CUDA
  * runtime call); make it before any stream capture.  The array is shared by
  * all calls and contexts in the process and keeps the last call's contents;
- * each call clears the part it uses.  Calls that overlap on the GPU race on
+ * each call writes the part it uses before it reads it.  Calls that overlap on the GPU race on
  * it: order them on one stream.  The call does not synchronize, so a
  * tensor-core completion wait that runs out in it (DMRG_PREC_BF16X3) is not
  * seen on return: dmrg_check_status reports it (DMRG_ETIMEOUT), as does the
@@ -440,9 +442,9 @@ int dmrg_batch_free(dmrg_batch *batch);
  * this many equal-work chunks), min_chunk (no chunk lighter than this many
  * FLOPs), tc_min (output blocks with a side >= tc_min and both sides <= 128
  * run on the tensor-core kernel in DMRG_PREC_BF16X3), by_work (1: chunks
- * launched heaviest first; 0: in output-block order), flat_wide (1: the
- * kernel for blocks of at most 32 x 32 runs one wide CTA per SM, 0: two
- * narrower CTAs per SM) and tc_tiny (the tensor-core kernel's shape: 1 = every
+ * launched heaviest first; 0: in output-block order), flat_wide (1: chunks of
+ * many tasks, or too few of them to fill the GPU, are shared by several groups
+ * of warps of a CTA; 0: one group of warps per chunk) and tc_tiny (the tensor-core kernel's shape: 1 = every
  * block with m <= 64 and q and every task's p <= 32 runs on the 32-column
  * shape, five CTAs per SM, in a launch of its own; 0 = that shape only when
  * every block fits it, else the 64- and 128-row shapes).  Defaults: 8192, 2e5,

@@ -359,14 +359,13 @@ struct ChainTune {
   int tc_min = 33;
   int by_work = 0;     // 1: launch groups heaviest first; 0: in output-block order (operand locality)
   int orient = 1;      // run each entry in its cheaper association (split task lists)
-  int flat_wide = 1;   // flat kernel CTAs: 1 = one wide CTA per SM (6 FP64 / 12 FP32 warps),
-                       // 0 = two narrower CTAs per SM (4 / 8 warps each)
+  int flat_wide = 1;   // CUDA-core kernels: 1 = several groups of warps may share a chunk, 0 = one per chunk
   int tc_tiny = 0;     // tensor-core kernel shapes: 1 = every block that fits the 32-column
                        // shape runs on it (a launch of its own), 0 = only when all blocks fit
 };
 // Host half of a task list's upload: the execution list (entries in their
 // cheaper association, cut into equal-work chunks when split_tasks), the launch
-// groups of the three chunk kernels (32 x 32 tiles, flattened lanes, tensor
+// groups of the chunk kernels (CUDA cores: blocks above and up to 32 x 32; tensor
 // cores) and the ordered reduction of the chunk slots.
 struct ExecPlan {
   std::vector<ChainEntry, NoInitAlloc<ChainEntry>> xs;
@@ -851,6 +850,47 @@ static void plan_tc(const std::vector<ChainEntry, NoInitAlloc<ChainEntry>> &xs, 
   if (entry_of) entry_of->swap(src);
 }
 
+// Operator images of more than this are given back before a renormalization allocates its block.
+static constexpr size_t kImagesKept = size_t(1) << 30;
+
+// The operators of a position as images (chain_pipe.cu): limbs of the FP64 operators and
+// temporaries, or their FP32 copies.
+struct OpSet {
+  DBuf<uint8_t> images;
+  std::vector<OpSlab> slabs;  // sorted by src once uploaded
+  DBuf<OpSlab> dslabs;
+  DBuf<int16_t> exps;
+  DBuf<int> id;  // slab of the identity of each dimension, or -1
+  int max_id = -1;
+  int64_t nblocks = 0;
+  bool ready = false, tried = false;
+  void release() {
+    images.release();
+    dslabs.release();
+    exps.release();
+    id.release();
+    slabs.clear();
+    max_id = -1;
+    nblocks = 0;
+    ready = tried = false;
+  }
+  size_t bytes() const { return images.n; }
+  OpTable table() const { return {dslabs.p, exps.p, id.p, (int)slabs.size(), max_id}; }
+  // the slabs to the device, sorted by source; the identities (src ~0) come last
+  void upload(cudaStream_t s) {
+    std::stable_sort(slabs.begin(), slabs.end(), [](const OpSlab &a, const OpSlab &b) { return a.src < b.src; });
+    max_id = -1;
+    for (const OpSlab &x : slabs)
+      if (x.src == ~0ull) max_id = std::max(max_id, x.rows);
+    std::vector<int> ids((size_t)max_id + 1, -1);
+    for (size_t i = 0; i < slabs.size(); ++i)
+      if (slabs[i].src == ~0ull) ids[(size_t)slabs[i].rows] = (int)i;
+    dslabs.upload(slabs, s);
+    id.upload(ids, s);
+    CK(cudaStreamSynchronize(s));  // ids is released
+  }
+};
+
 // A task list on the device.  When the tensor cores are enabled, output blocks
 // with both sides <= 128, one side >= tc_min and every entry's n, p <= 128 go
 // to the tensor-core kernel; of the rest, blocks of at most 32 x 32 go to the
@@ -862,7 +902,8 @@ static void plan_tc(const std::vector<ChainEntry, NoInitAlloc<ChainEntry>> &xs, 
 // thousands of independent tasks.
 struct DevChain {
   DBuf<ChainEntry> ent, xent;
-  DBuf<ChainGroup> all, big, flat;
+  DBuf<ChainGroup> all, cores;
+  DBuf<ChainItem> items;  // work items of the CUDA-core kernels, classes 4 to 0
   DBuf<ReduceGroup> red;
   DBuf<double> scratch;
   // tensor-core groups: entries with pre-split operand tiles (operators tiled
@@ -875,11 +916,57 @@ struct DevChain {
   int npts = 0, ntc_shape[3] = {0, 0, 0};
   int flat_wide = 1;
   int tc_tiny = 0;
-  int nall = 0, nbig = 0, nflat = 0, ntc = 0, ntiles = 0, nred = 0;
+  int nall = 0, ntc = 0, nred = 0;
+  int nitems[kChainClasses] = {};
+  PipeClass classes[kChainClasses];
+  int ncores = 0;
   int64_t nent = 0;
   int64_t red_total = 0, scratch_n = 0;
   bool split = false;
   bool ops32 = false;  // X and Z operands are FP32 copies (else the FP64 masters)
+  // prepared operands (H.psi lists): images of the operators, and per call those of psi
+  bool pipe = false;
+  const OpSet *ops = nullptr;
+  DBuf<PipeEntry> pent;
+  DBuf<PipeStack> stacks;
+  DBuf<int> nstacks, pexp;
+  DBuf<PsiSpan> spans;
+  DBuf<uint8_t> pimages;
+  int nspans = 0;
+  bool on_cores() const {
+    for (int n : nitems)
+      if (n > 0) return true;
+    return false;
+  }
+
+  // Run the list's CUDA-core chunks on prepared operands: o over the list's own operators, sp
+  // the psi blocks.
+  void prepare(const OpSet *o, std::vector<PsiSpan> sp, cudaStream_t s) {
+    pipe = false;
+    ops = o;
+    if (!on_cores() || !o || !o->ready || sp.size() >= (size_t(1) << 24)) return;
+    int64_t img = 0;
+    for (PsiSpan &b : sp) {
+      b.img = img;
+      img += pipe_image_size(ops32, b.rows, b.cols) + pipe_image_size(ops32, b.cols, b.rows);
+    }
+    if (img >= (int64_t(1) << 32)) return;
+    nspans = (int)sp.size();
+    spans.upload(sp, s);
+    pimages.alloc((size_t)std::max<int64_t>(img, 1) * (ops32 ? 4 : 8));
+    pexp.alloc(sp.size());
+    pent.alloc((size_t)nent);
+    stacks.alloc((size_t)nent);
+    nstacks.alloc((size_t)ncores + 1);  // and a flag after them
+    int *bad = nstacks.p + ncores;
+    CK(cudaMemsetAsync(bad, 0, sizeof(int), s));
+    CK(launch_pipe_entries(xent.p, cores.p, ncores, pent.p, stacks.p, nstacks.p, bad, o->table(), spans.p, nspans, ops32,
+                           s));
+    int is_bad = 0;
+    CK(cudaMemcpyAsync(&is_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));  // also: sp may be released
+    pipe = !is_bad;                // else the general kernels take the list
+  }
 
   void upload(const ChainList &CL, cudaStream_t s, bool tensor_cores = false, bool split_tasks = false,
               const ChainTune &tune = ChainTune(), bool ops32_in = false) {
@@ -890,23 +977,56 @@ struct DevChain {
     flat_wide = tune.flat_wide;
     tc_tiny = tune.tc_tiny;
     const auto &xs = X.xs;
-    const std::vector<ChainGroup> &vb = X.vb, &vf = X.vf, &vt = X.vt;
+    const std::vector<ChainGroup> &vt = X.vt;
     const std::vector<ReduceGroup> &vr = X.vr;
-    const int tiles = X.tiles;
     const int64_t soff = X.soff, e0 = X.e0;
     ent.upload(CL.flat, s);  // the task list as built (diagonal, batching)
     xent.upload(xs, s);      // the execution list of the chunk kernels
     nent = (int64_t)CL.flat.size();
     all.upload(CL.grp, s);
-    big.upload(vb, s);
-    flat.upload(vf, s);
+    // chunks of the CUDA-core kernels, cut into work items by kernel class
+    std::vector<ChainGroup> vc(X.vb);
+    vc.insert(vc.end(), X.vf.begin(), X.vf.end());
+    std::vector<int> pmax(vc.size(), 0), nmax(vc.size(), 0);
+    parallel_for((vc.size() + 63) / 64, [&](size_t c) {
+      for (size_t i = c * 64; i < std::min(vc.size(), (c + 1) * 64); ++i)
+        for (int j = vc[i].first; j < vc[i].first + vc[i].count; ++j) {
+          pmax[i] = std::max(pmax[i], xs[j].p);
+          nmax[i] = std::max(nmax[i], xs[j].n);
+        }
+    });
+    std::vector<ChainItem> vi[kChainClasses], iv;
+    for (PipeClass &c : classes) c = PipeClass();
+    for (int i = 0; i < (int)vc.size(); ++i) {
+      const int cls = chain_item_class(vc[i].m, vc[i].q, nmax[i], pmax[i]), cols = chain_item_cols(cls);
+      vc[i].tile0 = cls;
+      for (int r0 = 0; r0 < vc[i].m; r0 += 32)
+        for (int c0 = 0; c0 < vc[i].q; c0 += cols) {
+          vi[cls].push_back({i, r0, c0, 0});
+          classes[cls].tasks += vc[i].count;
+        }
+      PipeClass &c = classes[cls];
+      c.items = (int)vi[cls].size();
+      c.m = std::max(c.m, vc[i].m);
+      c.q = std::max(c.q, vc[i].q);
+      c.n = std::max(c.n, nmax[i]);
+      c.p = std::max(c.p, pmax[i]);
+    }
+    for (int cls = kChainClasses - 1; cls >= 0; --cls) {
+      // most tasks first: a chunk of many small tasks takes longest, and started last it would
+      // run on alone (results do not depend on the order)
+      std::stable_sort(vi[cls].begin(), vi[cls].end(),
+                       [&](const ChainItem &a, const ChainItem &b) { return vc[a.g].count > vc[b.g].count; });
+      nitems[cls] = (int)vi[cls].size();
+      iv.insert(iv.end(), vi[cls].begin(), vi[cls].end());
+    }
+    ncores = (int)vc.size();
+    cores.upload(vc, s);
+    items.upload(iv, s);
     build_tc(xs, vt, s);
     red.upload(vr, s);
     nall = (int)CL.grp.size();
-    nbig = (int)vb.size();
-    nflat = (int)vf.size();
     nred = (int)vr.size();
-    ntiles = tiles;
     red_total = e0;
     scratch_n = soff;
     if (split) scratch.alloc((size_t)std::max<int64_t>(soff, 1));
@@ -946,8 +1066,16 @@ struct DevChain {
     ent.release();
     xent.release();
     all.release();
-    big.release();
-    flat.release();
+    cores.release();
+    items.release();
+    pent.release();
+    stacks.release();
+    nstacks.release();
+    spans.release();
+    pexp.release();
+    pimages.release();
+    pipe = false;
+    ops = nullptr;
     red.release();
     scratch.release();
     tce.release();
@@ -956,7 +1084,8 @@ struct DevChain {
     optiles.release();
     psitiles.release();
     tc_counter.release();
-    nall = nbig = nflat = ntc = ntiles = nred = npts = 0;
+    nall = ntc = nred = npts = 0;
+    for (int &n : nitems) n = 0;
     ntc_shape[0] = ntc_shape[1] = ntc_shape[2] = 0;
     nent = red_total = scratch_n = 0;
   }
@@ -974,20 +1103,20 @@ struct DevChain {
   }
 
   // The launch sequence.  The chunk partials of a split task list go to the
-  // list's own scratch array, or to ext (at least scratch_n doubles, cleared
-  // here) when the caller provides one; nothing is allocated here.
+  // list's own scratch array, or to ext (at least scratch_n doubles) when the caller provides one; nothing is allocated here.
   void launch(uint64_t xb, uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s, int *status = nullptr,
               double *ext = nullptr) const {
     double *part = ext ? ext : scratch.p;
     const uint64_t tb = split ? (uint64_t)(uintptr_t)part : db;
-    if (split && scratch_n > 0) CK(cudaMemsetAsync(part, 0, scratch_n * sizeof(double), s));
-    if (ops32) {
-      CK(launch_chain_f32ops(xent.p, big.p, nbig, ntiles, xb, yb, zb, tb, s));
-      CK(launch_chain_flat_f32ops(xent.p, flat.p, nflat, xb, yb, zb, tb, s, flat_wide ? 12 : 8));
-    } else {
-      CK(launch_chain_fp64(xent.p, big.p, nbig, ntiles, xb, yb, zb, tb, s));
-      CK(launch_chain_flat_fp64(xent.p, flat.p, nflat, xb, yb, zb, tb, s, flat_wide ? 6 : 4));
-    }
+    if (pipe) {
+      const double *psi = reinterpret_cast<const double *>(yb);
+      CK(launch_psi_images(spans.p, nspans, psi, pimages.p, pexp.p, ops32, s));
+      const PipeArgs a{pent.p, stacks.p, nstacks.p, xent.p, cores.p, pimages.p, pexp.p, psi, tb};
+      CK(launch_chain_pipe(a, ops32, items.p, classes, flat_wide, s));
+    } else if (ops32)
+      CK(launch_chain_f32ops(xent.p, cores.p, items.p, nitems, xb, yb, zb, tb, s, flat_wide));
+    else
+      CK(launch_chain_fp64(xent.p, cores.p, items.p, nitems, xb, yb, zb, tb, s, flat_wide));
     launch_tc(yb, tb, status, s);
     if (split) CK(launch_reduce_partials(red.p, nred, red_total, part, (double *)(uintptr_t)db, s));
   }
@@ -1084,6 +1213,7 @@ struct HPlan {
   const DevBlock *lb = nullptr, *rb = nullptr;
   Psi psi;
   DevTemps temps;
+  OpSet ops;  // images of the FP64 operators
   DevChain chain;
   double flops = 0.0;
   long long ntasks = 0;
@@ -1091,6 +1221,7 @@ struct HPlan {
   // mixed precision: FP32 copies of the operators and temporaries + their task list
   bool lowp = false;
   DBuf<float> f32[4];  // left ops, right ops, left temps, right temps
+  OpSet ops32;         // images of them
   DevChain chain32;
 };
 
@@ -1376,6 +1507,79 @@ static void hpsi_chainlist(dmrg_ctx *c, bool f32, ChainList &CL, double &flops) 
   }
 }
 
+static std::vector<PsiSpan> psi_spans(const Psi &Y, int64_t shift = 0) {
+  std::vector<PsiSpan> v;
+  v.reserve(Y.blk.size());
+  for (const PsiBlock &b : Y.blk) v.push_back({b.off + shift, 0, b.ma, b.md});
+  return v;
+}
+
+// Images of the position's operators and temporaries (f32: of their FP32 copies), unless they
+// would take more than a third of the free device memory (the general kernels then convert as
+// they read).
+static void build_images(dmrg_ctx *c, bool f32) {
+  HPlan &P = c->plan;
+  OpSet &S = f32 ? P.ops32 : P.ops;
+  if (S.tried) return;
+  DevBlock *blk[2] = {lblock(c), rblock(c)};
+  const uint64_t esize = f32 ? 4 : 8;
+  S.slabs.clear();
+  S.nblocks = 0;
+  uint64_t need = 0;
+  auto slab = [&](uint64_t src, int rows, int cols, int K) {
+    if (K <= 0 || rows <= 0 || cols <= 0) return;
+    S.slabs.push_back({src, need, S.nblocks, rows, cols});
+    S.nblocks += K;
+    need += (uint64_t)K * (pipe_image_size(f32, rows, cols) + pipe_image_size(f32, cols, rows)) * esize;
+  };
+  const double *src64[4] = {blk[0]->arena(), blk[1]->arena(), P.temps.arena[0].p, P.temps.arena[1].p};
+  for (int i = 0; i < 4; ++i) {
+    const BlockLayout &b = blk[i & 1]->lay;
+    const void *base = f32 ? static_cast<const void *>(P.f32[i].p) : src64[i];
+    const uint64_t e0 = (uint64_t)(uintptr_t)base / esize;
+    auto family = [&](const std::vector<int> &bra, const std::vector<int64_t> &off, int64_t fbase, int K) {
+      for (int a = 0; a < (int)b.sec.size(); ++a)
+        if (bra[a] >= 0) slab(e0 + (uint64_t)(fbase + off[a]), b.sec[bra[a]].dim, b.sec[a].dim, K);
+    };
+    if (i < 2)
+      for (const Family &F : b.fam) family(F.bra, F.off, F.base, F.K());
+    else
+      for (const TempFamily &F : P.temps.set.fam[i & 1]) family(F.bra, F.off, F.base, F.K());
+  }
+  std::vector<char> has;
+  for (int i = 0; i < 2; ++i)
+    for (const Sector &sec : blk[i]->lay.sec) {
+      if ((int)has.size() <= sec.dim) has.resize((size_t)sec.dim + 1, 0);
+      if (!has[(size_t)sec.dim]) slab(~0ull, sec.dim, sec.dim, 1);
+      has[(size_t)sec.dim] = 1;
+    }
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  if (need > (free_b + S.images.n) / 3) {
+    S.release();
+    S.tried = true;
+    return;
+  }
+  S.images.alloc((size_t)std::max<uint64_t>(need, 1));
+  S.exps.alloc((size_t)std::max<int64_t>(S.nblocks, 1));
+  for (OpSlab &x : S.slabs) x.img += (uint64_t)(uintptr_t)S.images.p;
+  DBuf<OpSlab> by_block;  // in the order of the blocks, before they are sorted
+  by_block.upload(S.slabs, c->stream);
+  CK(launch_op_images(by_block.p, (int)S.slabs.size(), S.nblocks, S.exps.p, f32, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  S.upload(c->stream);
+  S.ready = true;
+  S.tried = true;
+}
+
+// The FP64 list on images (also made when a mixed-precision run first needs it).
+static void prepare_fp64(dmrg_ctx *c) {
+  HPlan &P = c->plan;
+  if (P.ops.tried && P.chain.ops == &P.ops) return;
+  build_images(c, false);
+  P.chain.prepare(&P.ops, psi_spans(P.psi), c->stream);
+}
+
 static void build_hplan(dmrg_ctx *c) {
   HPlan &P = c->plan;
   require_blocks(c);
@@ -1389,6 +1593,9 @@ static void build_hplan(dmrg_ctx *c) {
   P.psi = psi_layout(lb->lay, rb->lay, c->nu, c->nd);
   const Psi &Y = P.psi;
   P.temps.set = TempSet();
+  P.ops.ready = P.ops.tried = P.ops32.ready = P.ops32.tried = false;
+  P.chain.pipe = P.chain32.pipe = false;
+  P.chain.ops = P.chain32.ops = nullptr;
   P.rps = resolve_pieces(c->I, c->k, lb->lay, rb->lay, P.temps.set);
   const BlockLayout *lay[2] = {&lb->lay, &rb->lay};
   const double *stored[2] = {lb->arena(), rb->arena()};
@@ -1406,6 +1613,7 @@ static void build_hplan(dmrg_ctx *c) {
   CK(cudaMemsetAsync(P.diag.p, 0, Y.dim * sizeof(double), c->stream));
   CK(launch_diag_fp64(P.chain.ent.p, P.chain.all.p, P.chain.nall, 0, 0, P.diag.p, c->stream));
   P.lowp = c->prec != DMRG_PREC_FP64;
+  if (!P.lowp) prepare_fp64(c);
   if (c->prec == DMRG_PREC_FP32) {
     // FP32 working copies of every operand of the H.psi task list (Davidson matvecs)
     const double *src[4] = {lb->arena(), rb->arena(), P.temps.arena[0].p, P.temps.arena[1].p};
@@ -1418,6 +1626,8 @@ static void build_hplan(dmrg_ctx *c) {
     double fl32 = 0.0;
     hpsi_chainlist(c, true, CL32, fl32);
     P.chain32.upload(CL32, c->stream, false, true, c->tune, true);
+    build_images(c, true);
+    P.chain32.prepare(&P.ops32, psi_spans(Y), c->stream);
     CK(cudaStreamSynchronize(c->stream));
   } else if (c->prec == DMRG_PREC_BF16X3) {
     // the tensor-core list reads the FP64 masters: tiles are split straight from them, and
@@ -1426,6 +1636,10 @@ static void build_hplan(dmrg_ctx *c) {
     double flt = 0.0;
     hpsi_chainlist(c, false, CLt, flt);
     P.chain32.upload(CLt, c->stream, true, true, c->tune, false);
+    if (P.chain32.on_cores()) {
+      build_images(c, false);
+      P.chain32.prepare(&P.ops, psi_spans(Y), c->stream);
+    }
     CK(cudaStreamSynchronize(c->stream));
   }
   CK(cudaStreamSynchronize(c->stream));
@@ -1460,6 +1674,7 @@ static void fold_events(dmrg_ctx *c) {
 static void hpsi_dev(dmrg_ctx *c, const double *psi, double *sigma, bool fp64 = false) {
   HPlan &P = c->plan;
   const bool lowp = P.lowp && !fp64;
+  if (!lowp) prepare_fp64(c);
   CK(cudaMemsetAsync(sigma, 0, P.psi.dim * sizeof(double), c->stream));
   if (c->ev_used + 2 > 4096) fold_events(c);
   while (c->ev.size() < c->ev_used + 2) {
@@ -1934,11 +2149,18 @@ static void do_renormalize(dmrg_ctx *c, int direction, const int *kept_in, const
     Odev.alloc((size_t)std::max<int64_t>(tot, 1));
     if (tot) CK(cudaMemcpyAsync(Odev.p, O, tot * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   }
-  auto nb = renormalize_block(c, direction, enl, kept, Odev, Ooff);
   // keep the old psi for the prediction
   Psi oldlay = c->plan.valid ? c->plan.psi : Psi();
-  DBuf<double> oldpsi;
   const bool can_predict = (O == nullptr) && c->psi_valid && c->plan.valid;
+  if (c->plan.ops.bytes() + c->plan.ops32.bytes() > kImagesKept) {  // room for the new block: the move ends this plan anyway
+    CK(cudaStreamSynchronize(c->stream));
+    c->plan.valid = false;
+    ++c->plan_gen;
+    c->plan.ops.release();
+    c->plan.ops32.release();
+  }
+  auto nb = renormalize_block(c, direction, enl, kept, Odev, Ooff);
+  DBuf<double> oldpsi;
   if (can_predict) std::swap(oldpsi.p, c->psi.p), std::swap(oldpsi.n, c->psi.n);
   c->plan.valid = false;
   c->psi_valid = false;
@@ -2468,6 +2690,8 @@ extern "C" int dmrg_set_precision(dmrg_ctx *c, int precision) {
     c->plan.valid = false;  // task lists and low-precision copies are rebuilt on next use
     c->plan.chain32.release();  // the old working precision's copies, tiles and task list
     for (auto &f : c->plan.f32) f.release();
+    c->plan.ops.release();
+    c->plan.ops32.release();
     ++c->plan_gen;
   }
   API_END
@@ -3190,7 +3414,7 @@ extern "C" int dmrg_selftest_tcgen05(int N, int K, const float *A, const float *
 // partials of the split task list live in a fixed file-scope device array
 // instead of memory allocated per plan.  The array is shared by every call and
 // every context in the process and keeps the last call's contents; the call
-// clears the part it uses first.  Calls whose kernels overlap on the GPU
+// writes the part it uses before it reads it.  Calls whose kernels overlap on the GPU
 // (other streams, other host threads) race on it, so such callers must
 // order their calls on one stream or serialize them.
 // ---------------------------------------------------------------------------
@@ -3274,6 +3498,8 @@ struct dmrg_batch {
   dmrg::ChainTune tune;
   DevChain chain;
   DBuf<double> psi, sigma;
+  OpSet ops;  // tables over the contexts' operator images (the images stay theirs)
+  std::vector<PsiSpan> spans;
   double flops = 0.0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -3321,6 +3547,33 @@ static void batch_chainlist(const std::vector<dmrg_ctx *> &ctxs, ChainList &CL, 
   }
 }
 
+// The contexts' operator images as one set.
+static void batch_images(dmrg_batch *b, cudaStream_t s) {
+  OpSet &S = b->ops;
+  S.release();
+  const bool f32 = b->ctx[0]->prec == DMRG_PREC_FP32;
+  for (dmrg_ctx *c : b->ctx) {
+    if ((c->prec == DMRG_PREC_FP32) != f32) return;
+    build_images(c, f32);
+    const OpSet &L = f32 ? c->plan.ops32 : c->plan.ops;
+    if (!L.ready) return;  // memory: the batch converts as it reads
+    S.nblocks += L.nblocks;
+  }
+  S.exps.alloc((size_t)std::max<int64_t>(S.nblocks, 1));
+  int64_t first = 0;
+  for (dmrg_ctx *c : b->ctx) {
+    const OpSet &L = f32 ? c->plan.ops32 : c->plan.ops;
+    for (OpSlab x : L.slabs) {
+      x.first += first;
+      S.slabs.push_back(x);
+    }
+    CK(cudaMemcpyAsync(S.exps.p + first, L.exps.p, L.nblocks * sizeof(int16_t), cudaMemcpyDeviceToDevice, s));
+    first += L.nblocks;
+  }
+  S.upload(s);
+  S.ready = true;
+}
+
 extern "C" int dmrg_batch_create(int n, dmrg_ctx *const *ctxs, dmrg_batch **out) {
   API_BEGIN
   if (n < 1 || !ctxs || !out) throw Fail{DMRG_EINVAL, "bad arguments"};
@@ -3341,6 +3594,12 @@ extern "C" int dmrg_batch_create(int n, dmrg_ctx *const *ctxs, dmrg_batch **out)
   b->lowp = ctxs[0]->prec != DMRG_PREC_FP64;
   b->tc = ctxs[0]->prec == DMRG_PREC_BF16X3;
   b->chain.upload(CL, b->stream, b->tc, true, b->tune, ctxs[0]->prec == DMRG_PREC_FP32);
+  for (size_t i = 0; i < b->ctx.size(); ++i) {
+    const auto sp = psi_spans(b->ctx[i]->plan.psi, b->off[i]);
+    b->spans.insert(b->spans.end(), sp.begin(), sp.end());
+  }
+  if (b->chain.on_cores()) batch_images(b.get(), b->stream);
+  b->chain.prepare(&b->ops, b->spans, b->stream);
   b->psi.alloc((size_t)std::max<long long>(b->off.back(), 1));
   b->sigma.alloc((size_t)std::max<long long>(b->off.back(), 1));
   CK(cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking));
@@ -3449,10 +3708,12 @@ static double time_chain(const DevChain &ch, const double *x, double *y, int64_t
 // Coordinate search: split granularity first, then (tensor cores only) the
 // smallest output-block side routed to the tensor-core kernel.
 static ChainTune autotune_chain(const ChainList &CL, bool tc, bool ops32, const double *x, double *y, int64_t n,
-                                cudaStream_t s, int *status, int reps, ChainTune start, double &best_ms) {
+                                cudaStream_t s, int *status, int reps, ChainTune start, double &best_ms,
+                                const OpSet *ops, const std::vector<PsiSpan> &spans) {
   auto run = [&](const ChainTune &t) {
     DevChain ch;
     ch.upload(CL, s, tc, true, t, ops32);
+    ch.prepare(ops, spans, s);
     return time_chain(ch, x, y, n, s, status, reps);
   };
   ChainTune best = start;
@@ -3533,8 +3794,10 @@ extern "C" int dmrg_autotune(dmrg_ctx *c, int reps, double *best_ms, double *par
     x.alloc((size_t)std::max<int64_t>(n, 1));
     y.alloc((size_t)std::max<int64_t>(n, 1));
     CK(launch_fill_guess(x.p, n, 0x5eedull, c->stream));
+    const bool f32 = c->prec == DMRG_PREC_FP32;
+    build_images(c, f32);
     best = autotune_chain(CL, tc, c->prec == DMRG_PREC_FP32, x.p, y.p, n, c->stream, c->dstatus.p, reps, c->tune,
-                          ms);
+                          ms, f32 ? &P.ops32 : &P.ops, psi_spans(P.psi));
     CK(cudaStreamSynchronize(c->stream));
   }
   check_status(c);
@@ -3875,13 +4138,15 @@ extern "C" int dmrg_batch_autotune(dmrg_batch *b, int reps, double *best_ms, dou
   b->gen.clear();
   for (dmrg_ctx *c : b->ctx) b->gen.push_back(c->plan_gen);
   const int64_t n = b->off.back();
+  batch_images(b, b->stream);
   CK(launch_fill_guess(b->psi.p, n, 0x5eedull, b->stream));
   double ms = 0.0;
   ChainTune best = autotune_chain(CL, b->tc, b->ctx[0]->prec == DMRG_PREC_FP32, b->psi.p, b->sigma.p, n, b->stream,
-                                  b->ctx[0]->dstatus.p, reps, b->tune, ms);
+                                  b->ctx[0]->dstatus.p, reps, b->tune, ms, &b->ops, b->spans);
   check_status(b->ctx[0]);
   b->tune = best;
   b->chain.upload(CL, b->stream, b->tc, true, best, b->ctx[0]->prec == DMRG_PREC_FP32);
+  b->chain.prepare(&b->ops, b->spans, b->stream);
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   b->exec = nullptr;

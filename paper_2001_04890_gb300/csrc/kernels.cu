@@ -1,12 +1,7 @@
-// FP64 device kernels of the two-site QC-DMRG hot path (sm_103a).
+// FP64 device kernels of the two-site QC-DMRG hot path (sm_103a); the batched triple
+// products are in chain_kernels.cu and tc_kernels.cu.
 //
-// chain_fp64:   batched triple product D += sum_e f_e X_e Y_e Z_e over a task
-//               list grouped by output block (one CTA owns each 32x32 output
-//               tile, so accumulation is deterministic and needs no atomics).
-//               Used for H.psi (Sec. 2.2.1, Eq. dgemm: X = A_l, Y = psi^s,
-//               Z = A_r^T), for the renormalization O^T (A (x) o) O of
-//               Sec. 2.2.2 / Eq. renorm_mat (X = O^T, Y = A, Z = O) and for
-//               the density matrix psi psi^T of Sec. 2.1.
+// reduce_partials: adds the chunks of a split task list in chunk order.
 // lincomb_fp64: pre-summed operators (Sec. 2.2.3, Eq. presum) as a GEMM
 //               [K_out x K_src] x [K_src x block elements] per sector.
 // Davidson helpers, a round-robin parallel Jacobi eigensolver for the small subspace
@@ -28,277 +23,6 @@ void add_kernel_launches(long long n) { g_launches.fetch_add(n); }
 
 __device__ __forceinline__ const double *dptr(uint64_t base, uint64_t off) {
   return reinterpret_cast<const double *>(base + off * 8ull);
-}
-
-template <typename T>
-__device__ __forceinline__ const T *tptr(uint64_t base, uint64_t off) {
-  return reinterpret_cast<const T *>(base + off * sizeof(T));
-}
-
-// TX/TY/TZ: operand element types; TA: accumulation type; D is FP64.
-template <typename TX, typename TY, typename TZ, typename TA>
-__global__ void __launch_bounds__(256) chain_kernel(const ChainEntry *__restrict__ E,
-                                                    const ChainGroup *__restrict__ G, int ngroups,
-                                                    uint64_t xb, uint64_t yb, uint64_t zb,
-                                                    uint64_t db) {
-  __shared__ TA Xs[32][33];
-  __shared__ TA Ys[32][33];
-  __shared__ TA Ts[32][33];
-  __shared__ TA Zs[32][33];
-  const int tile = blockIdx.x;
-  int lo = 0, hi = ngroups - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (G[mid].tile0 <= tile) lo = mid; else hi = mid - 1;
-  }
-  const ChainGroup g = G[lo];
-  const int ntq = (g.q + 31) >> 5;
-  const int tl = tile - g.tile0;
-  const int r0 = (tl / ntq) * 32, c0 = (tl % ntq) * 32;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-  const int mrows = min(32, g.m - r0), qcols = min(32, g.q - c0);
-  TA acc[4] = {0, 0, 0, 0};
-
-  for (int ei = g.first; ei < g.first + g.count; ++ei) {
-    const ChainEntry e = E[ei];
-    const bool xid = e.x == IDN, yid = e.y == IDN, zid = e.z == IDN;
-    const TX *X = xid ? nullptr : tptr<TX>(xb, e.x);
-    const TY *Y = yid ? nullptr : tptr<TY>(yb, e.y);
-    const TZ *Z = zid ? nullptr : tptr<TZ>(zb, e.z);
-    const TA f = (TA)e.f;
-    const int n = e.n, p = e.p;
-    const int pbeg = zid ? c0 : 0;
-    const int pend = zid ? min(c0 + 32, p) : p;
-    for (int p0 = pbeg; p0 < pend; p0 += 32) {
-      const int pc = min(32, pend - p0);
-      TA t[4] = {0, 0, 0, 0};
-      if (xid || yid) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int r = ty + 8 * i;
-          if (r < mrows && tx < pc) {
-            const int64_t R = r0 + r, Cc = p0 + tx;
-            if (xid && yid) t[i] = (R == Cc) ? (TA)1 : (TA)0;
-            else if (xid) t[i] = (TA)Y[R * e.yrs + Cc * e.ycs];
-            else t[i] = (TA)X[R * e.xrs + Cc * e.xcs];
-          }
-        }
-      } else {
-        for (int n0 = 0; n0 < n; n0 += 32) {
-          const int nc = min(32, n - n0);
-          for (int idx = tid; idx < 1024; idx += 256) {
-            const int i = idx >> 5, kk = idx & 31;
-            Xs[i][kk] = (i < mrows && kk < nc)
-                            ? (TA)X[(int64_t)(r0 + i) * e.xrs + (int64_t)(n0 + kk) * e.xcs] : (TA)0;
-            Ys[i][kk] = (i < nc && kk < pc)
-                            ? (TA)Y[(int64_t)(n0 + i) * e.yrs + (int64_t)(p0 + kk) * e.ycs] : (TA)0;
-          }
-          __syncthreads();
-          if (tx < pc) {
-            for (int kk = 0; kk < nc; ++kk) {
-              const TA y = Ys[kk][tx];
-#pragma unroll
-              for (int i = 0; i < 4; ++i)
-                if (ty + 8 * i < mrows) t[i] = fma(Xs[ty + 8 * i][kk], y, t[i]);
-            }
-          }
-          __syncthreads();
-        }
-      }
-      if (zid) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = fma(f, t[i], acc[i]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) Ts[ty + 8 * i][tx] = t[i];
-        for (int idx = tid; idx < 1024; idx += 256) {
-          const int kk = idx >> 5, j = idx & 31;
-          Zs[kk][j] = (kk < pc && j < qcols)
-                          ? (TA)Z[(int64_t)(p0 + kk) * e.zrs + (int64_t)(c0 + j) * e.zcs] : (TA)0;
-        }
-        __syncthreads();
-        if (tx < qcols) {
-          TA sacc[4] = {0, 0, 0, 0};
-          for (int kk = 0; kk < pc; ++kk) {
-            const TA z = Zs[kk][tx];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (ty + 8 * i < mrows) sacc[i] = fma(Ts[ty + 8 * i][kk], z, sacc[i]);
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) acc[i] = fma(f, sacc[i], acc[i]);
-        }
-        __syncthreads();
-      }
-    }
-  }
-  double *D = const_cast<double *>(tptr<double>(db, g.d));
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = ty + 8 * i;
-    if (r < mrows && tx < qcols) D[(int64_t)(r0 + r) * g.drs + (int64_t)(c0 + tx) * g.dcs] += (double)acc[i];
-  }
-}
-
-// Output blocks of at most 32 x 32: one warp per (output block, entry chunk);
-// lanes are assigned to the m*p elements of T = X Y and the m*q elements of
-// the output block in flattened order, so a lane is idle only in the last
-// partial round (no 32-wide padding of small sector blocks).  Four elements
-// per lane are advanced together for instruction-level parallelism.
-template <typename TX, typename TY, typename TZ, typename TA, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS) chain_flat_kernel(const ChainEntry *__restrict__ E,
-                                                               const ChainGroup *__restrict__ G,
-                                                               int ngroups, uint64_t xb, uint64_t yb,
-                                                               uint64_t zb, uint64_t db) {
-  extern __shared__ __align__(16) unsigned char flat_smem[];
-  TA *base = reinterpret_cast<TA *>(flat_smem);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gi = blockIdx.x * WARPS + warp;
-  if (gi >= ngroups) return;  // warp-uniform; only warp barriers below
-  // three 32 x 33 tiles per warp; the Z tile reuses the X tile once T is formed
-  TA(*Xs)[33] = reinterpret_cast<TA(*)[33]>(base + (size_t)warp * 3 * 32 * 33);
-  TA(*Ys)[33] = Xs + 32;
-  TA(*Ts)[33] = Xs + 64;
-  TA(*Zs)[33] = Xs;
-  const ChainGroup g = G[gi];
-  const int m = g.m, q = g.q, mq = m * q;
-  TA acc[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) acc[j] = 0;
-  for (int ei = g.first; ei < g.first + g.count; ++ei) {
-    const ChainEntry e = E[ei];
-    const bool xid = e.x == IDN, yid = e.y == IDN, zid = e.z == IDN;
-    const TX *X = xid ? nullptr : tptr<TX>(xb, e.x);
-    const TY *Y = yid ? nullptr : tptr<TY>(yb, e.y);
-    const TZ *Z = zid ? nullptr : tptr<TZ>(zb, e.z);
-    const TA f = (TA)e.f;
-    const int n = e.n, p = e.p;
-    for (int p0 = 0; p0 < p; p0 += 32) {
-      const int pc = min(32, p - p0);
-      const int mp = m * pc;
-      // ---- T (m x pc) into Ts
-      if (xid || yid) {
-        for (int t = lane; t < mp; t += 32) {
-          const int i = t / pc, c = t % pc;
-          TA v;
-          if (xid && yid) v = (i == p0 + c) ? (TA)1 : (TA)0;
-          else if (xid) v = (TA)Y[(int64_t)i * e.yrs + (int64_t)(p0 + c) * e.ycs];
-          else v = (TA)X[(int64_t)i * e.xrs + (int64_t)(p0 + c) * e.xcs];
-          Ts[i][c] = v;
-        }
-      } else {
-        for (int t = lane; t < mp; t += 32) Ts[t / pc][t % pc] = 0;
-        for (int n0 = 0; n0 < n; n0 += 32) {
-          const int nc = min(32, n - n0);
-          for (int t = lane; t < m * nc; t += 32) {
-            const int i = t / nc, kk = t % nc;
-            Xs[i][kk] = (TA)X[(int64_t)i * e.xrs + (int64_t)(n0 + kk) * e.xcs];
-          }
-          for (int t = lane; t < nc * pc; t += 32) {
-            const int kk = t / pc, c = t % pc;
-            Ys[kk][c] = (TA)Y[(int64_t)(n0 + kk) * e.yrs + (int64_t)(p0 + c) * e.ycs];
-          }
-          __syncwarp();
-          // element t = b0 + 32 u + lane; rounds of four warp-wide element groups
-          for (int b0 = 0; b0 < mp; b0 += 128) {
-            const int nu = min(4, (mp - b0 + 31) >> 5);  // warp-uniform
-            int ii[4], cc[4];
-            TA s4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int t = min(b0 + 32 * u + lane, mp - 1);
-              ii[u] = t / pc;
-              cc[u] = t % pc;
-              s4[u] = 0;
-            }
-            for (int kk = 0; kk < nc; ++kk) {
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-                if (u < nu) s4[u] = fma(Xs[ii[u]][kk], Ys[kk][cc[u]], s4[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              if (b0 + 32 * u + lane < mp) Ts[ii[u]][cc[u]] += s4[u];
-          }
-          __syncwarp();
-        }
-      }
-      __syncwarp();
-      // ---- acc += f T Z (or f T when Z is the identity)
-      if (zid) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int t = lane + 32 * j;
-          if (t < mq) {
-            const int i = t / q, c = t % q;
-            if (c >= p0 && c < p0 + pc) acc[j] = fma(f, Ts[i][c - p0], acc[j]);
-          }
-        }
-      } else {
-        for (int t = lane; t < pc * q; t += 32) {
-          const int kk = t / q, c = t % q;
-          Zs[kk][c] = (TA)Z[(int64_t)(p0 + kk) * e.zrs + (int64_t)c * e.zcs];
-        }
-        __syncwarp();
-#pragma unroll
-        for (int j0 = 0; j0 < 32; j0 += 4) {
-          const int nu = min(4, (mq - 32 * j0 + 31) >> 5);  // warp-uniform
-          if (nu <= 0) break;
-          int ii[4], cc[4];
-          TA s4[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int t = min(lane + 32 * (j0 + u), mq - 1);
-            ii[u] = t / q;
-            cc[u] = t % q;
-            s4[u] = 0;
-          }
-          for (int kk = 0; kk < pc; ++kk) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              if (u < nu) s4[u] = fma(Ts[ii[u]][kk], Zs[kk][cc[u]], s4[u]);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) acc[j0 + u] = fma(f, s4[u], acc[j0 + u]);
-        }
-      }
-      __syncwarp();
-    }
-  }
-  double *D = const_cast<double *>(tptr<double>(db, g.d));
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const int t = lane + 32 * j;
-    if (t < mq) D[(int64_t)(t / q) * g.drs + (int64_t)(t % q) * g.dcs] += (double)acc[j];
-  }
-}
-
-template <typename TX, typename TY, typename TZ, typename TA, int WARPS>
-static cudaError_t launch_flat_w(const ChainEntry *e, const ChainGroup *g, int ngroups, uint64_t xb,
-                                 uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s) {
-  const int smem = WARPS * 3 * 32 * 33 * (int)sizeof(TA);
-  auto kern = chain_flat_kernel<TX, TY, TZ, TA, WARPS>;
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (err != cudaSuccess) return err;
-  COUNT(1);
-  kern<<<(ngroups + WARPS - 1) / WARPS, 32 * WARPS, smem, s>>>(e, g, ngroups, xb, yb, zb, db);
-  return cudaGetLastError();
-}
-
-// warps per CTA: FP64 6 (one CTA per SM) or 4 (two CTAs, 8 warps per SM);
-// FP32 12 (one CTA) or 8 (two CTAs, 16 warps per SM)
-cudaError_t launch_chain_flat_fp64(const ChainEntry *e, const ChainGroup *g, int ngroups, uint64_t xb,
-                                   uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s, int warps) {
-  if (ngroups <= 0) return cudaSuccess;
-  if (warps == 4) return launch_flat_w<double, double, double, double, 4>(e, g, ngroups, xb, yb, zb, db, s);
-  return launch_flat_w<double, double, double, double, 6>(e, g, ngroups, xb, yb, zb, db, s);
-}
-
-cudaError_t launch_chain_flat_f32ops(const ChainEntry *e, const ChainGroup *g, int ngroups, uint64_t xb,
-                                     uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s, int warps) {
-  if (ngroups <= 0) return cudaSuccess;
-  if (warps == 8) return launch_flat_w<float, double, float, float, 8>(e, g, ngroups, xb, yb, zb, db, s);
-  return launch_flat_w<float, double, float, float, 12>(e, g, ngroups, xb, yb, zb, db, s);
 }
 
 // out[ red.d + ...] += sum over the task chunks of their partial blocks, in chunk order
@@ -327,22 +51,6 @@ cudaError_t launch_reduce_partials(const ReduceGroup *r, int nred, int64_t total
   if (blocks > 152 * 32) blocks = 152 * 32;
   COUNT(1);
   reduce_partials_kernel<<<(int)blocks, 256, 0, s>>>(r, nred, total, scratch, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_chain_fp64(const ChainEntry *e, const ChainGroup *g, int ngroups, int ntiles,
-                              uint64_t xb, uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s) {
-  if (ngroups <= 0 || ntiles <= 0) return cudaSuccess;
-  COUNT(1);
-  chain_kernel<double, double, double, double><<<ntiles, 256, 0, s>>>(e, g, ngroups, xb, yb, zb, db);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_chain_f32ops(const ChainEntry *e, const ChainGroup *g, int ngroups, int ntiles,
-                                uint64_t xb, uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s) {
-  if (ngroups <= 0 || ntiles <= 0) return cudaSuccess;
-  COUNT(1);
-  chain_kernel<float, double, float, float><<<ntiles, 256, 0, s>>>(e, g, ngroups, xb, yb, zb, db);
   return cudaGetLastError();
 }
 

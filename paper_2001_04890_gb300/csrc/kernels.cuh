@@ -25,17 +25,109 @@ struct DevStatus {
   int error;
 };
 
-cudaError_t launch_chain_fp64(const ChainEntry *e, const ChainGroup *g, int ngroups, int ntiles,
-                              uint64_t xb, uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s);
+// Work item of the CUDA-core kernels: the rows from r0 and columns from c0 of one group's output
+// block, as many as the item's class takes (chain_item_class: 16 x 16, 16 x 32, 32 x 32, 32 x 64,
+// 32 x 96, 32 x 128).
+struct ChainItem {
+  int g, r0, c0, pad;
+};
+constexpr int kChainClasses = 6;
+int chain_item_class(int m, int q, int nmax, int pmax);  // largest n, p of the group's tasks
+int chain_item_cols(int cls);
+// D = sum over each group's tasks (written, not added).  items: those of class 5, then 4, 3, 2, 1, 0,
+// count[class] of each.  wide: chunks that do not fill the GPU are shared by several warps.
+cudaError_t launch_chain_fp64(const ChainEntry *e, const ChainGroup *g, const ChainItem *items, const int *count,
+                              uint64_t xb, uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s, int wide = 1);
 // same task list with FP32 operators X, Z (FP64 psi in, FP64 sigma out, FP32 accumulation)
-cudaError_t launch_chain_f32ops(const ChainEntry *e, const ChainGroup *g, int ngroups, int ntiles,
-                                uint64_t xb, uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s);
-// one warp per output block of at most 32 x 32, lanes over flattened elements
-// warps per CTA: FP64 6 or 4, FP32 12 or 8 (other values: the first)
-cudaError_t launch_chain_flat_fp64(const ChainEntry *e, const ChainGroup *g, int ngroups, uint64_t xb,
-                                   uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s, int warps = 6);
-cudaError_t launch_chain_flat_f32ops(const ChainEntry *e, const ChainGroup *g, int ngroups, uint64_t xb,
-                                     uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s, int warps = 12);
+cudaError_t launch_chain_f32ops(const ChainEntry *e, const ChainGroup *g, const ChainItem *items, const int *count,
+                                uint64_t xb, uint64_t yb, uint64_t zb, uint64_t db, cudaStream_t s, int wide = 1);
+
+// Prepared operands of H.psi (chain_pipe.cu): images of the operator blocks (limbs of the FP64
+// operators, or FP32) and of the psi blocks.
+struct OpSlab {   // blocks of equal shape, one after the other (the operators of one sector transition)
+  uint64_t src;   // element address of the first block (~0: an identity)
+  uint64_t img;   // byte address of its images: of the block, then of its transpose
+  int64_t first;  // number of the slab's first block
+  int rows, cols;
+};
+struct OpTable {
+  const OpSlab *s = nullptr;  // sorted by src
+  const int16_t *exps = nullptr;
+  const int *id = nullptr;    // slab of the identity of each dimension up to max_id, or -1
+  int n = 0, max_id = -1;
+};
+struct PsiSpan {
+  int64_t off, img;  // element offset of the block in psi, and of its images among the images
+  int rows, cols;
+};
+struct PipeEntry {
+  uint64_t x, z;  // byte addresses of the images of X (rows: its rows) and Z (rows: its columns)
+  double f;
+  int w;          // limbs: sum of the exponents of X, Z and f (INT_MIN: the task needs FP64)
+  int src;        // the task in the execution list
+};
+static_assert(sizeof(PipeEntry) == 32, "PipeEntry is 32 bytes");
+struct PipeStack {
+  int e;          // first entry
+  uint16_t n, p;  // Y is n x p
+  uint32_t y;     // element offset of its image (rows: its columns)
+  unsigned yb : 24, ns : 4, flags : 4;  // psi block, tasks, 1: no scaling of T, 2: needs FP64
+};
+static_assert(sizeof(PipeStack) == 16, "the kernel reads a PipeStack as one vector");
+constexpr int kPipeMaxN = 120;  // inner dimension that 64-bit sums of limb products take
+constexpr int kPipeTile = 592;  // elements of the X, Y and Z tiles of the kernel for small blocks
+// Tasks on one psi block that run as one stack: what the tiles of the class's kernel hold (rows of
+// X, depth of T).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int pipe_stack_cap(bool fx, int cls, int m, int q, int n, int p) {
+  if (cls > 1 || n > 32 || p > 32) return 1;
+  const bool small = cls == 0;
+  const int pn = fx ? ((n + 1) >> 2 << 2) + 2 : ((n + 3) >> 3 << 3) + 4;
+  const int pp = fx ? ((p + 1) >> 2 << 2) + 2 : ((p + 3) >> 3 << 3) + 4;
+  const int pt = fx ? (p + 1) & ~1 : (p + 3) & ~3;
+  int c = 32 / pt;
+  const int rows = (small ? 32 : 16) / m;
+  if (rows < c) c = rows;
+  if (small) {
+    if (kPipeTile / (m * pn) < c) c = kPipeTile / (m * pn);
+    if (kPipeTile / (q * pp) < c) c = kPipeTile / (q * pp);
+  } else if (32 / q < c) {
+    c = 32 / q;
+  }
+  return c < 1 ? 1 : c < 8 ? c : 8;
+}
+int64_t pipe_image_size(bool f32, int rows, int cols);  // elements of one image
+// images and exponents of every block; s in block order
+cudaError_t launch_op_images(const OpSlab *s, int nslabs, int64_t nblocks, int16_t *exps, bool f32, cudaStream_t st);
+cudaError_t launch_psi_images(const PsiSpan *b, int nblocks, const double *psi, void *out, int *exps, bool f32,
+                              cudaStream_t st);
+// The tasks of every group (tile0: its kernel class) as PipeEntry and their stacks (from the
+// group's first entry on; nstacks per group); limbs: sorted by psi block within the group.  *bad is set if a task has a form that
+// the kernel does not take.
+cudaError_t launch_pipe_entries(const ChainEntry *e, const ChainGroup *g, int ngroups, PipeEntry *out,
+                                PipeStack *stacks, int *nstacks, int *bad, const OpTable &ops, const PsiSpan *b,
+                                int nblocks, bool f32, cudaStream_t st);
+struct PipeArgs {
+  const PipeEntry *e;
+  const PipeStack *stacks;
+  const int *nstacks;
+  const ChainEntry *tasks;  // the execution list (FP64 operators: for tasks that fixed point does not take)
+  const ChainGroup *g;
+  const void *psi;          // images of the psi blocks
+  const int *pexp;          // limbs: their exponents
+  const double *psi64;      // the call's psi
+  uint64_t db;
+};
+struct PipeClass {  // the items of a kernel class
+  int items = 0;
+  int64_t tasks = 0;
+  int m = 0, q = 0, n = 0, p = 0;  // largest dimensions
+};
+// as launch_chain_fp64 / launch_chain_f32ops (f32), on prepared operands
+cudaError_t launch_chain_pipe(const PipeArgs &a, bool f32, const ChainItem *items, const PipeClass *classes, int wide,
+                              cudaStream_t s);
 
 // Split task lists: every output block's entries are cut into chunks whose
 // partial blocks go to a scratch buffer; this adds them in chunk order.

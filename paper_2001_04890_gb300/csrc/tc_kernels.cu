@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(T2_THREADS, CTAS) chain_tc2_kernel(const TcEnt
         if (R >= 0 && R < m) {
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            if (c0 + i < q) Dout[(int64_t)R * g.drs + (int64_t)(c0 + i) * g.dcs] += (double)v[i];
+            if (c0 + i < q) Dout[(int64_t)R * g.drs + (int64_t)(c0 + i) * g.dcs] = (double)v[i];
         }
       }
       tc::fence_before();
