@@ -260,15 +260,6 @@ __device__ __forceinline__ void carry(Arith<true>::Acc &x) {
 __device__ __forceinline__ void carry(float &) {}
 __device__ __forceinline__ unsigned magnitude(long long t) { return (unsigned)((t ^ (t >> 63)) >> 32); }
 
-// t (fh 2^31 + fl) 2^-62 for |t| < 2^62, |fh|, |fl| < 2^31
-__device__ __forceinline__ long long mul_coef(long long t, int fh, int fl) {
-  const int th = (int)(t >> 31), tl = (int)((unsigned)t & 0x7fffffffu);
-  const long long mid = (long long)th * fl + (long long)tl * fh;
-  return (long long)th * fh + (mid >> 31);
-}
-
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-
 // f 2^e for an f whose exponent is moderate (|e| stays below 1000, see tile_special)
 __device__ __forceinline__ double scaled(double f, int e) {
   return __hiloint2double(__double2hiint(f) + (e << 20), __double2loint(f));

@@ -164,7 +164,10 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
           const int mid = (lo + hi + 1) >> 1;
           if (B[mid].off <= y) lo = mid; else hi = mid - 1;
         }
-        k = (unsigned long long)lo << 32 | (unsigned)i;
+        // limbs: tasks with a coefficient other than +-2^k run alone
+        const double f = E[g.first + b0 + i].f;
+        const bool alone = FX && ((__double2hiint(f) & 0xfffff) != 0 || __double2loint(f) != 0);
+        k = (unsigned long long)(2 * lo + (alone ? 1 : 0)) << 32 | (unsigned)i;
       }
       key[i] = k;
     }
@@ -207,7 +210,8 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
       bool head = false;
       PipeStack st{};
       if (i < cnt) {
-        const int yb = (int)(key[i] >> 32);
+        const int yb = (int)(key[i] >> 33);
+        const bool alone = (key[i] >> 32) & 1;
         const ChainEntry e = E[g.first + b0 + (int)(unsigned)key[i]];
         const bool xt = e.xcs != 1 || (e.xrs == 1 && e.n > 1), yt = e.ycs != 1 || (e.yrs == 1 && e.p > 1),
                    zt = e.zcs != 1 || (e.zrs == 1 && g.q > 1);
@@ -252,7 +256,7 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
         if (FX && (ef > 1023 + 100 || ef < 1023 - 100)) ex = -1;  // a coefficient that needs FP64
         p.w = FX ? (ex < 0 || ez < 0 ? INT_MIN : ex + ez + ef) : 0;
         p.src = g.first + b0 + (int)(unsigned)key[i];
-        const int cap = pipe_stack_cap(FX, g.tile0, g.m, g.q, e.n, e.p);
+        const int cap = alone ? 1 : pipe_stack_cap(FX, g.tile0, g.m, g.q, e.n, e.p);
         head = (i - run0[i]) % cap == 0;
         st.e = g.first + b0 + i;
         st.ns = min(cap, run1[i] - i + 1);
@@ -283,21 +287,14 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
     }
   }
   if (tid == 0) nstacks[blockIdx.x] = ns;
-  // stacks whose members share one weight and have coefficients +-2^k need no scaling of T;
-  // stacks with a member that fixed point does not take are marked
-  if (FX) {
+  if (FX) {  // stacks with a member that fixed point does not take are marked
     __threadfence_block();
     __syncthreads();
     for (int i = tid; i < ns; i += 256) {
       PipeStack &st = stacks[g.first + i];
-      bool plain = true, special = false;
-      const int w = out[st.e].w;
-      for (int j = 0; j < st.ns; ++j) {
-        const PipeEntry &p = out[st.e + j];
-        special |= p.w == INT_MIN;
-        plain = plain && p.w == w && (__double2hiint(p.f) & 0xfffff) == 0 && __double2loint(p.f) == 0;
-      }
-      st.flags = (uint8_t)((plain ? 1 : 0) | (special ? 2 : 0));
+      bool special = false;
+      for (int j = 0; j < st.ns; ++j) special |= out[st.e + j].w == INT_MIN;
+      st.flags = special ? 1 : 0;
     }
   }
 }
@@ -313,6 +310,7 @@ template <int N>
 __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+__device__ __forceinline__ void prefetch(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 // n bytes (a multiple of 16) by the threads tid of nthr
 __device__ __forceinline__ void copy_run(void *dst, const void *src, int n, int tid, int nthr) {
 #pragma unroll 1
@@ -347,44 +345,6 @@ struct PipeSmem {
   int x, b, pt, group;
 };
 
-// Sums of stage 1 under one scale: coefficients multiplied in, members shifted to the largest
-// weight.  Only for stacks whose members differ in weight or have coefficients other than
-// +-2^k (one-site terms), or whose sums span several chunks.
-template <int N>
-__device__ __noinline__ int scale_sums(Arith<true>::Acc (&acc)[N], const PipeEntry *E, int ns, int s1, int na, int nb,
-                                       int NB, int pc, int rows, float invm, int4 *mypar) {
-  const int lane = threadIdx.x & 31, lr = lane >> 3, lc = lane & 7;
-  const int w = lane < ns ? E[lane].w : INT_MIN;
-  const int wmax = __reduce_max_sync(kFull, w);
-  if (lane < ns) {
-    const double f = E[lane].f;
-    const unsigned long long fm =
-        ((unsigned long long)((__double2hiint(f) & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(f)) << 9;
-    const int sg = __double2hiint(f) < 0 ? -1 : 1;  // f = sg (fh 2^31 + fl) 2^-61, fh in [2^30, 2^31)
-    mypar[lane] = make_int4(sg * (int)(fm >> 31), sg * (int)((unsigned)fm & 0x7fffffffu), min(wmax - w, 63), 0);
-  }
-  __syncwarp();
-  unsigned mx = 0;
-#pragma unroll 1
-  for (int i = 0; i < N; ++i) {
-    const int a = i / NB, b = i - a * NB, row = lr + 4 * a;
-    if (a >= na || b >= nb) continue;
-    const int4 pr = mypar[ns > 1 ? min(small_div(row, invm), ns - 1) : 0];
-    long long t = mul_coef(fold(acc[i], 0) >> s1, pr.x, pr.y) >> pr.z;
-    if (lc + 8 * b >= pc || row >= rows) t = 0;
-    acc[i].hh = t;
-    mx = max(mx, magnitude(t));
-  }
-  mx = __reduce_max_sync(kFull, mx);
-  const int rsh = max(0, 7 - __clz(mx | 1));  // below 2^57
-#pragma unroll 1
-  for (int i = 0; i < N; ++i) {
-    if (rsh) acc[i].hh = (acc[i].hh + (1ll << (rsh - 1))) >> rsh;
-    acc[i].cr = 0;
-  }
-  return wmax - E[0].w + s1 + 1 + rsh;  // weight of the new sums against the old ones' hh
-}
-
 // The stacks of an item that fixed point does not take, in FP64 from the operators; added to
 // the item's output, which the kernel has written.
 __device__ __noinline__ void slow_stacks(const PipeEntry *P, const PipeStack *S, int nst, const ChainEntry *E,
@@ -394,7 +354,7 @@ __device__ __noinline__ void slow_stacks(const PipeEntry *P, const PipeStack *S,
   const int tid = threadIdx.x, nthr = blockDim.x;
   double *D = reinterpret_cast<double *>(db + g.d * 8ull);
   for (int st = 0; st < nst; ++st) {
-    if (!(S[st].flags & 2) && pexp[S[st].yb] >= 0) continue;
+    if (!S[st].flags && pexp[S[st].yb] >= 0) continue;
     for (int i = S[st].e; i < S[st].e + S[st].ns; ++i) {
       const ChainEntry e = E[P[i].src];
       const bool xi = e.x == ~0ull, zi = e.z == ~0ull;
@@ -441,7 +401,8 @@ __device__ __noinline__ void slow_stacks(const PipeEntry *P, const PipeStack *S,
 //
 // The X of a stack's tasks lie below one another in the X tile, so stage 1 is one product with
 // the Y that they share; their parts of T lie beside one another, and stage 2 sums over them.
-// For that the parts of T have one scale, with the tasks' coefficients multiplied in.
+// For that the parts of T get one scale, coefficients +-2^k and all; a task with another
+// coefficient (a one-site term) is a stack of its own.
 template <bool FX, bool SMALL, int WC>
 __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShape<FX, SMALL, WC>::MINB)
     chain_pipe_kernel(const PipeEntry *__restrict__ E, const PipeStack *__restrict__ stacks,
@@ -457,7 +418,6 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
   constexpr int NA = S::NA, NB = S::NB, CW = S::CW, PI = S::PI, VK = A::VK, ES = (int)sizeof(Elem);
   extern __shared__ __align__(16) unsigned char pipe_smem[];
   __shared__ int te[8][WC];   // exponents of the T tiles
-  __shared__ int4 par[8][8];  // per warp and stack member: coefficient (two limbs), shift
   const int gthr = 32 * wr * WC;
   const int grp = WC == 1 ? (int)threadIdx.x / gthr : 0, ngrp = WC == 1 ? (int)blockDim.x / gthr : 1;
   const int tid = (int)threadIdx.x - grp * gthr, warp = tid >> 5, lane = tid & 31;
@@ -487,95 +447,108 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
   // most 32 x 32, running on for larger ones
   const bool apart = !FX && gm <= 32 && gq <= 32;
 
-  // a unit: chunk c of stage 1 or (two) of stage 2 of a stack, columns of T from p0
-  struct Unit {
-    int e, ns, n, p, ey, flags;
-    uint32_t y;
-    int p0, c;
-    bool two;
+  // A stack (PipeStack as read, and the exponent of its Y).  It is read one stack ahead, and
+  // what it points to is asked for in time, so that no copy waits for a chain of loads.
+  struct Stack {
+    int4 d;
+    int ey;
+    __device__ __forceinline__ int e() const { return d.x; }
+    __device__ __forceinline__ int n() const { return d.y & 0xffff; }
+    __device__ __forceinline__ int p() const { return (int)((unsigned)d.y >> 16); }
+    __device__ __forceinline__ uint32_t y() const { return (uint32_t)d.z; }
+    __device__ __forceinline__ int yb() const { return d.w & 0xffffff; }
+    __device__ __forceinline__ int ns() const { return (d.w >> 24) & 15; }
+    __device__ __forceinline__ bool special() const { return (unsigned)d.w >> 28 || ey < 0; }
   };
   int si = grp;
-  auto next_stack = [&](Unit &u) {  // false: no further stack of this group
-    for (; si < nst; si += ngrp) {
-      const int4 s = *reinterpret_cast<const int4 *>(stk + si);  // PipeStack
-      u.e = s.x;
-      u.n = s.y & 0xffff;
-      u.p = (int)((unsigned)s.y >> 16);
-      u.y = (uint32_t)s.z;
-      u.ns = (s.w >> 24) & 15;
-      u.flags = (int)((unsigned)s.w >> 28);
-      u.ey = 0;
-      u.p0 = u.c = 0;
-      u.two = false;
-      if (FX) {
-        u.ey = pexp[s.w & 0xffffff];
-        if (u.ey < 0 || (u.flags & 2)) {
-          any_special = true;
-          continue;
-        }
-      }
-      si += ngrp;
-      return true;
-    }
-    return false;
+  auto member = [&](int ns) { return ns <= 1 ? 0 : tid >> (5 - (32 - __clz(ns - 1))); };  // stacks: one warp
+  auto take = [&](Stack &t) {  // ns() = 0: no further stack of this group
+    t.d = si < nst ? *reinterpret_cast<const int4 *>(stk + si) : make_int4(0, 0, 0, 0);
+    t.ey = 0;
+    si += ngrp;
   };
-  auto chunks1 = [&](const Unit &u) { return (u.n + KD - 1) / KD; };
-  auto advance = [&](Unit &u) {
-    ++u.c;
-    if (!u.two) {
-      if (u.c < chunks1(u)) return true;
-      u.c = 0;
-      u.two = true;
-      return true;
-    }
-    if (WC > 1 && u.c < min(WC, (u.p - u.p0 + CW - 1) / CW)) return true;
-    u.c = 0;
-    u.two = false;
-    u.p0 += CW * WC;
-    if (u.p0 < u.p) return true;
-    return next_stack(u);
+  auto ask = [&](Stack &t) {  // for the exponent of Y and this thread's share of the entries
+    if (t.ns() == 0) return;
+    if (FX) t.ey = pexp[t.yb()];
+    prefetch(E + t.e() + min(member(t.ns()), t.ns() - 1));
   };
-  // copy a unit's tiles; the group's threads are split over the stack's members
-  auto copy_unit = [&](const Unit &u, Elem *B) {
-    const int lg = u.ns <= 1 ? 0 : 32 - __clz(u.ns - 1);
-    const int mem = lg ? tid >> (5 - lg) : 0, sub = gthr >> lg, st = lg ? tid & (sub - 1) : tid;  // stacks: one warp
-    const int k0 = u.two ? u.p0 + u.c * CW : u.c * KD;          // summed index
-    const int K = u.two ? u.p : u.n, w = min(KD, K - k0), P = pitch_of<FX>(w);
-    const int R = u.two ? gq : gm, r0 = u.two ? it.c0 : it.r0, rows = u.two ? qi : mi;
-    if (mem < u.ns) {
-      const PipeEntry &e = E[u.e + mem];
-      const char *img = reinterpret_cast<const char *>(u.two ? e.z : e.x);
-      Elem *dst = (u.two ? B : Xs) + mem * rows * P;
-      copy_run(dst, img + ((int64_t)(k0 / KD) * R * PI + r0 * P) * ES, rows * P * ES, st, sub);
+  auto skip_special = [&](Stack &t) {
+    while (FX && t.ns() > 0 && t.special()) {
+      any_special = true;
+      take(t);
+      ask(t);
     }
-    if (!u.two)
-      copy_run(B, psi + u.y + (int64_t)(k0 / KD) * u.p * PI + u.p0 * P, min(CW * WC, u.p - u.p0) * P * ES, tid, gthr);
+  };
+  // Copy the tiles of a unit of t: chunk c of stage 1 or (two) of stage 2, columns of T from p0.
+  auto copy_unit = [&](const Stack &t, int p0, int c, bool two, Elem *B) {
+    const int ns = t.ns(), lg = ns <= 1 ? 0 : 32 - __clz(ns - 1), mem = lg ? tid >> (5 - lg) : 0, sub = gthr >> lg,
+              st = lg ? tid & (sub - 1) : tid;
+    const int k0 = two ? p0 + c * CW : c * KD;  // summed index
+    const int w = min(KD, (two ? t.p() : t.n()) - k0), P = pitch_of<FX>(w);
+    const int R = two ? gq : gm, r0 = two ? it.c0 : it.r0, rows = two ? qi : mi;
+    if (mem < ns) {
+      const PipeEntry &e = E[t.e() + mem];
+      copy_run((two ? B : Xs) + mem * rows * P,
+               reinterpret_cast<const char *>(two ? e.z : e.x) + ((int64_t)(k0 / KD) * R * PI + r0 * P) * ES, rows * P * ES,
+               st, sub);
+    }
+    if (!two)
+      copy_run(B, psi + t.y() + (int64_t)(k0 / KD) * t.p() * PI + p0 * P, min(CW * WC, t.p() - p0) * P * ES, tid, gthr);
     cp_commit();
   };
 
-  Unit u;
-  bool more = next_stack(u);
+  Stack u, nx;  // the stack at hand and the next one
+  take(u);
+  ask(u);
+  skip_special(u);
+  if (u.ns() > 0) {
+    copy_unit(u, 0, 0, false, Bs);
+    take(nx);
+  }
+  int p0 = 0, c = 0;
+  bool two = false;
   int par_b = 0;  // buffer of the current unit
-  if (more) copy_unit(u, Bs);
   Acc acc[NA][NB];
 #pragma unroll 1
-  while (more) {
-    Unit v = u;
-    const bool next = advance(v);
+  while (u.ns() > 0) {
+    const int nch = (u.n() + KD - 1) / KD;
+    // the unit after this one
+    int vp = p0, vc = c + 1;
+    bool vtwo = two, over = false;
+    if (!two) {
+      if (vc >= nch) {
+        vc = 0;
+        vtwo = true;
+      }
+    } else if (WC == 1 || vc >= min(WC, (u.p() - p0 + CW - 1) / CW)) {
+      vc = 0;
+      vtwo = false;
+      vp += CW * WC;
+      if (vp >= u.p()) {
+        vp = 0;
+        over = true;
+      }
+    }
     cp_wait<0>();
     group_sync(grp, gthr);  // the tiles are here, the unit before this one has been computed
-    const bool late = next && !u.two && !v.two;  // X is still in use: copied after this unit
-    if (next && !late) copy_unit(v, Bs + (par_b ^ 1) * sm.b);
+    const bool late = !over && !two && !vtwo;  // X is still in use: copied after this unit
+    if (!two && c == 0 && p0 == 0) ask(nx);
+    if (over) {
+      skip_special(nx);
+      if (nx.ns() > 0) copy_unit(nx, 0, 0, false, Bs + (par_b ^ 1) * sm.b);
+    } else if (!late) {
+      copy_unit(u, vp, vc, vtwo, Bs + (par_b ^ 1) * sm.b);
+    }
     const Elem *B = Bs + par_b * sm.b;
-    const int ns = u.ns;
-    const int pc = min(CW, u.p - u.p0 - CW * (u.two ? u.c : wcol));  // columns of the T tile at hand
+    const int ns = u.ns();
+    const int pc = min(CW, u.p() - p0 - CW * (two ? c : wcol));  // columns of the T tile at hand
     const int pt = (pc + VK - 1) / VK * VK;                          // a member's columns in the tile
-    const bool busy = m > 0 && (u.two ? q : pc) > 0;
-    const int rows = u.two ? m : ns * m, na = (rows + 3) >> 2, nb = ((u.two ? q : pc) + 7) >> 3;
+    const bool busy = m > 0 && (two ? q : pc) > 0;
+    const int rows = two ? m : ns * m, na = (rows + 3) >> 2, nb = ((two ? q : pc) + 7) >> 3;
     if (busy) {
       // ---- sums of the unit: X Y, or over the members of T Z
-      const int kc = u.two ? pc : min(KD, u.n - u.c * KD), P = pitch_of<FX>(kc);
-      if (u.two || u.c == 0 || apart) {
+      const int kc = two ? pc : min(KD, u.n() - c * KD), P = pitch_of<FX>(kc);
+      if (two || c == 0 || apart) {
 #pragma unroll
         for (int a = 0; a < NA; ++a)
 #pragma unroll
@@ -586,14 +559,14 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
 #pragma unroll
           for (int b = 0; b < NB; ++b) carry(acc[a][b]);
       }
-      const Elem *Ar = u.two ? Ts + u.c * 16 * PT + lr * PT : Xs + (rw * wrow + lr) * P;
+      const Elem *Ar = two ? Ts + c * 16 * PT + lr * PT : Xs + (rw * wrow + lr) * P;
       const Elem *Br = B + (wcol * CW + lc) * P;
 #pragma unroll 1
-      for (int mem = 0; mem < (u.two ? ns : 1); ++mem, Ar += pt, Br += qi * P) {
-        mm_any(Ar, u.two ? PT : P, Br, P, kc, na, nb, acc);
+      for (int mem = 0; mem < (two ? ns : 1); ++mem, Ar += pt, Br += qi * P) {
+        mm_any(Ar, two ? PT : P, Br, P, kc, na, nb, acc);
         if constexpr (!FX) {
-          if (u.two) {  // D += f (T Z), task by task
-            const float f = (float)E[u.e + mem].f;
+          if (two) {  // D += f (T Z), task by task
+            const float f = (float)E[u.e() + mem].f;
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -605,9 +578,12 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
         }
       }
     }
-    if (busy && u.two) {
+    if (busy && two) {
       if constexpr (FX) {  // D += 2^e (sums)
-        const double sc = pow2(58 - 1 + (WC > 1 ? tex[u.c] : tex[0]));
+        // a single task's coefficient is applied here; those of a stack are +-2^k and are in T
+        const double f1 = ns == 1 ? E[u.e()].f : 1.0;
+        const int e2 = 58 - 1 + (WC > 1 ? tex[c] : tex[0]);
+        const double sc = __hiloint2double((__double2hiint(f1) & 0x800fffff) | ((e2 + 1023) << 20), __double2loint(f1));
 #pragma unroll
         for (int a = 0; a < 4; ++a)
           if (a < na) {
@@ -617,57 +593,46 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
           }
       }
     } else if (busy) {
-      if (apart || u.c == chunks1(u) - 1) {
+      if (apart || c == nch - 1) {
         Elem *T = Ts + wcol * 16 * PT + lc;
         const float invm = 1.0f / (float)m;
         if constexpr (FX) {
-          int eT = E[u.e].w + u.ey - 2158 - 1023 - 1079;
-          unsigned neg = 0;  // members with a negative coefficient
-          const bool plain = (u.flags & 1) && u.n <= KD;
-          if (plain) {
-            neg = __ballot_sync(kFull, lane < ns && __double2hiint(E[u.e + min(lane, ns - 1)].f) < 0);
-          } else {
-            Acc tmp[NA * NB];
-#pragma unroll
-            for (int a = 0; a < NA; ++a)
-#pragma unroll
-              for (int b = 0; b < NB; ++b) tmp[a * NB + b] = acc[a][b];
-            eT += scale_sums<NA * NB>(tmp, E + u.e, ns, u.n <= KD ? 0 : 2, na, nb, NB, pc, rows, invm,
-                                      par[threadIdx.x >> 5]);
-#pragma unroll
-            for (int a = 0; a < NA; ++a)
-#pragma unroll
-              for (int b = 0; b < NB; ++b) acc[a][b] = tmp[a * NB + b];
-          }
+          // the members' weights below the largest one (bits 0-5) and signs (bit 8): their parts
+          // of T get one scale
+          const int w = lane < ns ? E[u.e() + lane].w : INT_MIN;
+          const int wmax = __reduce_max_sync(kFull, w);
+          int below = 0;
+          if (ns > 1 && lane < ns) below = min(wmax - w, 62) | (__double2hiint(E[u.e() + lane].f) < 0 ? 256 : 0);
           unsigned mx = 0;
 #pragma unroll
           for (int a = 0; a < NA; ++a)
             if (a < na) {
+              const int row = lr + 4 * a, sh = ns > 1 ? __shfl_sync(kFull, below, small_div(row, invm)) & 63 : 0;
 #pragma unroll
               for (int b = 0; b < NB; ++b) {
-                const unsigned h = magnitude(acc[a][b].hh);
-                mx = max(mx, b < nb && lc + 8 * b < pc && lr + 4 * a < rows ? h : 0u);
+                const unsigned h = sh < 32 ? magnitude(acc[a][b].hh) >> sh : 0u;
+                mx = max(mx, b < nb && lc + 8 * b < pc && row < rows ? h : 0u);
               }
             }
           mx = __reduce_max_sync(kFull, mx);
-          const int bits = 64 - __clz(mx | 1);  // |hh| < 2^bits
-          const int lsh = max(0, 57 - bits), rsh = max(0, bits - 57);  // T = (hh << lsh) + cross, >> rsh
-          eT += 58 - lsh + rsh;
-          if (lane == 0) tex[WC > 1 ? wcol : 0] = eT;
-          const long long half = 1ll << (28 - lsh), rhalf = rsh ? 1ll << (rsh - 1) : 0;
+          const int up = __clz(mx | 1) - 7;  // T = hh 2^(up - sh) + cross, below 2^57
+          if (lane == 0) tex[WC > 1 ? wcol : 0] = wmax + u.ey - 2158 - 1023 - 1079 + 58 - up;
+          const bool down = ns > 1 || up < 0;
 #pragma unroll
           for (int a = 0; a < NA; ++a) {
             if (a < na) {
               const int row = lr + 4 * a, mem = ns > 1 ? small_div(row, invm) : 0;
+              const int v = ns > 1 ? __shfl_sync(kFull, below, mem) : 0;
+              const int net = up - (v & 63), l = max(net, 0), r = max(-net, 0);
+              const long long half = 1ll << (28 - l), rhalf = (1ll << r) >> 1, sg = -(long long)(v >> 8);
               Elem *Tr = T + (row - mem * m) * PT + mem * pt;
-              const long long sg = -(long long)((neg >> mem) & 1);
               if (row < rows) {
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
                   if (lc + 8 * b < pt) {
-                    long long t = (acc[a][b].hh << lsh) + ((acc[a][b].cr + half) >> (29 - lsh));
-                    if (rsh) t = (t + rhalf) >> rsh;
-                    Tr[8 * b] = lc + 8 * b < pc ? limbs((t ^ sg) - sg) : Elem();
+                    long long t = (acc[a][b].hh << l) + ((acc[a][b].cr + half) >> (29 - l));
+                    if (down) t = (((t + rhalf) >> r) ^ sg) - sg;
+                    Tr[8 * b] = lc + 8 * b < pc ? limbs(t) : Elem();
                   }
                 }
               }
@@ -683,7 +648,7 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
 #pragma unroll
                 for (int b = 0; b < NB; ++b)
                   if (lc + 8 * b < pt)
-                    Tr[8 * b] = lc + 8 * b < pc ? (apart && u.c > 0 ? Tr[8 * b] + acc[a][b] : acc[a][b]) : 0.f;
+                    Tr[8 * b] = lc + 8 * b < pc ? (apart && c > 0 ? Tr[8 * b] + acc[a][b] : acc[a][b]) : 0.f;
               }
             }
           }
@@ -692,11 +657,16 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
     }
     if (late) {
       group_sync(grp, gthr);
-      copy_unit(v, Bs + (par_b ^ 1) * sm.b);
+      copy_unit(u, vp, vc, vtwo, Bs + (par_b ^ 1) * sm.b);
     }
     par_b ^= 1;
-    u = v;
-    more = next;
+    p0 = vp;
+    c = vc;
+    two = vtwo;
+    if (over) {
+      u = nx;
+      if (u.ns() > 0) take(nx);
+    }
   }
   if constexpr (WC == 1) {
     if (ngrp > 1) {  // the groups' sums, added in group order
@@ -773,7 +743,8 @@ cudaError_t launch_pipe(const PipeArgs &a, const ChainItem *items, const PipeCla
 }
 
 template <bool FX>
-cudaError_t launch_pipe_all(const PipeArgs &a, const ChainItem *items, const PipeClass *c, bool wide, cudaStream_t s) {
+cudaError_t launch_pipe_all(const PipeArgs &a, const ChainItem *items, const PipeClass *c, bool wide, cudaStream_t s,
+                            cudaStream_t s1, cudaStream_t s2) {
   cudaError_t err;
   auto next = [&](int cls) {
     const ChainItem *p = items;
@@ -781,20 +752,20 @@ cudaError_t launch_pipe_all(const PipeArgs &a, const ChainItem *items, const Pip
     return p;
   };
   const ChainItem *i5 = next(5), *i4 = next(4), *i3 = next(3), *i2 = next(2), *i1 = next(1), *i0 = next(0);
-  if ((err = launch_pipe<FX, false, 4>(a, i5, c[5], 2, false, s)) != cudaSuccess) return err;
+  if ((err = launch_pipe<FX, false, 4>(a, i5, c[5], 2, false, s1)) != cudaSuccess) return err;
   if ((err = launch_pipe<FX, false, 3>(a, i4, c[4], 2, false, s)) != cudaSuccess) return err;
-  if ((err = launch_pipe<FX, false, 2>(a, i3, c[3], 2, false, s)) != cudaSuccess) return err;
+  if ((err = launch_pipe<FX, false, 2>(a, i3, c[3], 2, false, s1)) != cudaSuccess) return err;
   if ((err = launch_pipe<FX, false, 1>(a, i2, c[2], 2, wide, s)) != cudaSuccess) return err;
-  if ((err = launch_pipe<FX, false, 1>(a, i1, c[1], 1, wide, s)) != cudaSuccess) return err;
-  return launch_pipe<FX, true, 1>(a, i0, c[0], 1, wide, s);
+  if ((err = launch_pipe<FX, false, 1>(a, i1, c[1], 1, wide, s1)) != cudaSuccess) return err;
+  return launch_pipe<FX, true, 1>(a, i0, c[0], 1, wide, s2);
 }
 
 }  // namespace
 
 cudaError_t launch_chain_pipe(const PipeArgs &a, bool f32, const ChainItem *items, const PipeClass *classes, int wide,
-                              cudaStream_t s) {
-  return f32 ? launch_pipe_all<false>(a, items, classes, wide != 0, s)
-             : launch_pipe_all<true>(a, items, classes, wide != 0, s);
+                              cudaStream_t s, cudaStream_t s1, cudaStream_t s2) {
+  return f32 ? launch_pipe_all<false>(a, items, classes, wide != 0, s, s1, s2)
+             : launch_pipe_all<true>(a, items, classes, wide != 0, s, s1, s2);
 }
 
 int64_t pipe_image_size(bool f32, int rows, int cols) {

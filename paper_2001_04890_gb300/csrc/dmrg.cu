@@ -891,6 +891,42 @@ struct OpSet {
   }
 };
 
+// Two streams beside a caller's, for the kernels of one launch sequence that do not depend on
+// one another: fork() orders them after the work queued on the caller's stream, join() orders
+// the caller's stream after them, so that to the caller everything happened on its stream.
+struct SideStreams {
+  cudaStream_t s[2] = {nullptr, nullptr};
+  cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
+  SideStreams() = default;
+  SideStreams(const SideStreams &) = delete;
+  SideStreams &operator=(const SideStreams &) = delete;
+  ~SideStreams() {
+    for (cudaStream_t x : s)
+      if (x) {
+        cudaStreamSynchronize(x);
+        cudaStreamDestroy(x);
+      }
+    for (cudaEvent_t e : ev)
+      if (e) cudaEventDestroy(e);
+  }
+  void create() {
+    for (cudaStream_t &x : s)
+      if (!x) CK(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
+    for (cudaEvent_t &e : ev)
+      if (!e) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  }
+  void fork(cudaStream_t main) const {
+    CK(cudaEventRecord(ev[0], main));
+    for (cudaStream_t x : s) CK(cudaStreamWaitEvent(x, ev[0], 0));
+  }
+  void join(cudaStream_t main) const {
+    for (int i = 0; i < 2; ++i) {
+      CK(cudaEventRecord(ev[1 + i], s[i]));
+      CK(cudaStreamWaitEvent(main, ev[1 + i], 0));
+    }
+  }
+};
+
 // A task list on the device.  When the tensor cores are enabled, output blocks
 // with both sides <= 128, one side >= tc_min and every entry's n, p <= 128 go
 // to the tensor-core kernel; of the rest, blocks of at most 32 x 32 go to the
@@ -933,6 +969,8 @@ struct DevChain {
   DBuf<PsiSpan> spans;
   DBuf<uint8_t> pimages;
   int nspans = 0;
+  SideStreams side;  // for the kernels of several classes
+  bool forked() const { return pipe && side.s[0]; }
   bool on_cores() const {
     for (int n : nitems)
       if (n > 0) return true;
@@ -966,6 +1004,9 @@ struct DevChain {
     CK(cudaMemcpyAsync(&is_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));  // also: sp may be released
     pipe = !is_bad;                // else the general kernels take the list
+    int kernels = ntc > 0 ? 1 : 0;
+    for (int n : nitems) kernels += n > 0;
+    if (pipe && kernels > 1) side.create();
   }
 
   void upload(const ChainList &CL, cudaStream_t s, bool tensor_cores = false, bool split_tasks = false,
@@ -1112,12 +1153,21 @@ struct DevChain {
       const double *psi = reinterpret_cast<const double *>(yb);
       CK(launch_psi_images(spans.p, nspans, psi, pimages.p, pexp.p, ops32, s));
       const PipeArgs a{pent.p, stacks.p, nstacks.p, xent.p, cores.p, pimages.p, pexp.p, psi, tb};
-      CK(launch_chain_pipe(a, ops32, items.p, classes, flat_wide, s));
-    } else if (ops32)
-      CK(launch_chain_f32ops(xent.p, cores.p, items.p, nitems, xb, yb, zb, tb, s, flat_wide));
-    else
-      CK(launch_chain_fp64(xent.p, cores.p, items.p, nitems, xb, yb, zb, tb, s, flat_wide));
-    launch_tc(yb, tb, status, s);
+      // the classes' kernels and the tensor-core ones write slots of their own: run side by side,
+      // each one's last CTAs leave room for the next one's first
+      const bool f = forked();
+      if (f) side.fork(s);
+      cudaStream_t s1 = f ? side.s[0] : s, s2 = f ? side.s[1] : s;
+      CK(launch_chain_pipe(a, ops32, items.p, classes, flat_wide, s, s1, s2));
+      launch_tc(yb, tb, status, s2);
+      if (f) side.join(s);
+    } else {
+      if (ops32)
+        CK(launch_chain_f32ops(xent.p, cores.p, items.p, nitems, xb, yb, zb, tb, s, flat_wide));
+      else
+        CK(launch_chain_fp64(xent.p, cores.p, items.p, nitems, xb, yb, zb, tb, s, flat_wide));
+      launch_tc(yb, tb, status, s);
+    }
     if (split) CK(launch_reduce_partials(red.p, nred, red_total, part, (double *)(uintptr_t)db, s));
   }
 };

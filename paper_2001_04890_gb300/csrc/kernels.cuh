@@ -71,7 +71,7 @@ struct PipeStack {
   int e;          // first entry
   uint16_t n, p;  // Y is n x p
   uint32_t y;     // element offset of its image (rows: its columns)
-  unsigned yb : 24, ns : 4, flags : 4;  // psi block, tasks, 1: no scaling of T, 2: needs FP64
+  unsigned yb : 24, ns : 4, flags : 4;  // psi block, tasks, whether one of them needs FP64
 };
 static_assert(sizeof(PipeStack) == 16, "the kernel reads a PipeStack as one vector");
 constexpr int kPipeMaxN = 120;  // inner dimension that 64-bit sums of limb products take
@@ -125,9 +125,10 @@ struct PipeClass {  // the items of a kernel class
   int64_t tasks = 0;
   int m = 0, q = 0, n = 0, p = 0;  // largest dimensions
 };
-// as launch_chain_fp64 / launch_chain_f32ops (f32), on prepared operands
+// as launch_chain_fp64 / launch_chain_f32ops (f32), on prepared operands; classes 2 and 4 run on s,
+// 1, 3 and 5 on s1, 0 on s2 (the caller orders them; all may be s)
 cudaError_t launch_chain_pipe(const PipeArgs &a, bool f32, const ChainItem *items, const PipeClass *classes, int wide,
-                              cudaStream_t s);
+                              cudaStream_t s, cudaStream_t s1, cudaStream_t s2);
 
 // Split task lists: every output block's entries are cut into chunks whose
 // partial blocks go to a scratch buffer; this adds them in chunk order.
