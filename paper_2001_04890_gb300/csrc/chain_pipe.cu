@@ -326,17 +326,22 @@ __device__ __forceinline__ void group_sync(int id, int nthr) {
     asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "r"(nthr) : "memory");
 }
 
-// Group shapes.  SMALL: output blocks of at most 16 x 16 whose tasks have p <= 16; a warp's
-// stage-1 tile is 32 rows (the stacked X of a stack) x 16 columns.  Else a warp has 16 rows x
-// 32 columns in both stages.
+// Group shapes.  A warp has 16 rows.  SMALL: output blocks of at most 16 x 16 and tasks whose X,
+// Y and Z fit kPipeTile, 16 columns a warp; else 32 columns.
+//
+// Threads an SM holds of the kernel for small blocks.  At 512 a lane's 128 registers do not hold
+// the limb sums, two stacks' descriptions and the addresses; measured at 384 / 512: H psi, 8
+// orbitals, M 64: 196 / 216 us; 16 vectors, 24 orbitals, M 512: 13.4 / 12.8 ms; Davidson, 10
+// orbitals, M 128: 157 / 168 ms.
+constexpr int kSmallThreads = 384;
 template <bool FX, bool SMALL, int WC>
 struct PipeShape {
-  static constexpr int NA = SMALL ? 8 : 4;  // rows per lane, stage 1
+  static constexpr int NA = 4;              // rows per lane
   static constexpr int NB = SMALL ? 2 : 4;  // columns per lane
   static constexpr int CW = 8 * NB;         // columns of a warp
   static constexpr int PI = pitch_of<FX>(KD);  // row pitch of a whole chunk
   static constexpr int MAXTHREADS = WC == 1 ? 128 : 64 * WC;
-  static constexpr int MINB = (WC == 4 ? 256 : 384) / MAXTHREADS;
+  static constexpr int MINB = (SMALL ? kSmallThreads : WC == 4 ? 256 : 384) / MAXTHREADS;
 };
 
 // Shared memory of a group (elements): the X tile, each of the two Y / Z buffers, and the T tiles
@@ -711,7 +716,7 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
 // when the others are done, and so are chunks that alone would not fill the GPU.
 int groups_per_item(int n, int64_t tasks, int wr, int resident) {
   int k = 1;
-  while (32 * wr * k < 128 && ((long long)n * wr * k < resident || tasks > 64ll * k * n)) k *= 2;
+  while (32 * wr * k < 128 && ((long long)n * wr * k < resident || tasks > 16ll * k * n)) k *= 2;
   return k;
 }
 
@@ -728,11 +733,11 @@ cudaError_t launch_pipe(const PipeArgs &a, const ChainItem *items, const PipeCla
   sm.x = SMALL ? kPipeTile : wr == 1 ? 16 * pitch(c.n) : mx * pitch(c.n);
   sm.b = SMALL ? kPipeTile : std::max(px * pitch(c.n), (wr == 1 ? 32 : qx) * pitch(c.p));
   sm.pt = WC == 1 && c.p > 16 ? pitch(c.p) : pitch(KD);
-  if (SMALL || wr == 1) sm.pt = pitch(KD);
+  if (wr == 1) sm.pt = pitch(SMALL ? 16 : KD);
   sm.group = sm.x + 2 * sm.b + wr * WC * 16 * sm.pt;
   sm.group = std::max(sm.group, 32 * wr * WC * (4 * S::NB + 1));  // the exchange of the groups' sums
   const int bytes = sm.group * (int)sizeof(Elem);
-  const int groups = share && FX ? groups_per_item(c.items, c.tasks, wr, 12 * 152) : 1;
+  const int groups = share && FX ? groups_per_item(c.items, c.tasks, wr, (SMALL ? kSmallThreads / 32 : 12) * 152) : 1;
   auto kern = chain_pipe_kernel<FX, SMALL, WC>;
   const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
   if (err != cudaSuccess) return err;

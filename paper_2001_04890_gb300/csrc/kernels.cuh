@@ -75,7 +75,7 @@ struct PipeStack {
 };
 static_assert(sizeof(PipeStack) == 16, "the kernel reads a PipeStack as one vector");
 constexpr int kPipeMaxN = 120;  // inner dimension that 64-bit sums of limb products take
-constexpr int kPipeTile = 592;  // elements of the X, Y and Z tiles of the kernel for small blocks
+constexpr int kPipeTile = 320;  // elements of the X, Y and Z tiles of the kernel for small blocks
 // Tasks on one psi block that run as one stack: what the tiles of the class's kernel hold (rows of
 // X, depth of T).
 #ifdef __CUDACC__
@@ -87,8 +87,8 @@ inline int pipe_stack_cap(bool fx, int cls, int m, int q, int n, int p) {
   const int pn = fx ? ((n + 1) >> 2 << 2) + 2 : ((n + 3) >> 3 << 3) + 4;
   const int pp = fx ? ((p + 1) >> 2 << 2) + 2 : ((p + 3) >> 3 << 3) + 4;
   const int pt = fx ? (p + 1) & ~1 : (p + 3) & ~3;
-  int c = 32 / pt;
-  const int rows = (small ? 32 : 16) / m;
+  int c = (small ? 16 : 32) / pt;
+  const int rows = 16 / m;
   if (rows < c) c = rows;
   if (small) {
     if (kPipeTile / (m * pn) < c) c = kPipeTile / (m * pn);
