@@ -179,13 +179,32 @@ __global__ void dots_stage1(const double *__restrict__ V, int k, int64_t n,
     for (int j = 0; j < 32; ++j)
       if (j < k) s[j] = fma(V[(int64_t)j * n + e], we, s[j]);
   }
-  // warp reduce
+  // Warp sums, every column's by the same tree (lane i + lane i + 16, then + 8, ...).  Up to six
+  // columns each by itself; more of them two at a time per step: half of the lanes add one
+  // column's pairs and half another's, so 31 additions serve 32 columns instead of 160 (an FP64
+  // addition takes a warp 64 clocks here: 37 us of a 16,600-element dot product of 1 to 25
+  // columns was these).
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (k <= 6) {
 #pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    double x = s[j];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if (lane == 0) red[warp][j] = x;
+    for (int j = 0; j < 6; ++j) {
+      if (j < k) {
+        double x = s[j];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        if (lane == 0) red[warp][j] = x;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+      for (int j = 0; j < o; ++j) {  // columns j (lower lanes) and j + o (upper lanes)
+        const bool up = lane & o;
+        const double give = up ? s[j] : s[j + o], keep = up ? s[j + o] : s[j];
+        s[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+    red[warp][lane] = s[0];  // lane's bits select its column
   }
   __syncthreads();
   if (threadIdx.x < k) {
