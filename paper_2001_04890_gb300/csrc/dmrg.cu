@@ -1021,10 +1021,10 @@ struct DevChain {
     const std::vector<ChainGroup> &vt = X.vt;
     const std::vector<ReduceGroup> &vr = X.vr;
     const int64_t soff = X.soff, e0 = X.e0;
-    ent.upload(CL.flat, s);  // the task list as built (diagonal, batching)
+    if (split) ent.upload(CL.flat, s);  // the task list as built (H.psi: diagonal, batching)
     xent.upload(xs, s);      // the execution list of the chunk kernels
     nent = (int64_t)CL.flat.size();
-    all.upload(CL.grp, s);
+    if (split) all.upload(CL.grp, s);
     // chunks of the CUDA-core kernels, cut into work items by kernel class
     std::vector<ChainGroup> vc(X.vb);
     vc.insert(vc.end(), X.vf.begin(), X.vf.end());

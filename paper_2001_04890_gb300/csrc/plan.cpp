@@ -2,6 +2,11 @@
 // See plan.hpp for the paper references.
 #include "plan.hpp"
 
+#include <unistd.h>
+
+#include <chrono>
+#include <condition_variable>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -15,6 +20,113 @@
 #include <utility>
 
 namespace dmrg {
+
+// ---------------------------------------------------------------- helper threads
+
+namespace {
+
+unsigned helper_count() { return std::max(1u, std::min(16u, std::thread::hardware_concurrency())) - 1; }
+
+// The helpers and the loop they work on.  A loop is open while its indices last; helpers join it
+// under the mutex, and the caller waits only for those that joined.
+struct Helpers {
+  std::atomic<bool> running{false};  // a loop has the helpers
+  std::mutex mu;
+  std::condition_variable wake, done;
+  unsigned alive = 0, joined = 0;
+  unsigned long long round = 0;
+  bool open = false;
+  size_t n = 0;
+  void (*call)(void *, size_t) = nullptr;
+  void *ctx = nullptr;
+  std::atomic<size_t> next{0};
+  const long process = (long)getpid();
+
+  void work() {
+    for (size_t i = next.fetch_add(1); i < n; i = next.fetch_add(1)) call(ctx, i);
+  }
+  void helper() {
+    std::unique_lock<std::mutex> lk(mu);
+    for (unsigned long long seen = 0;;) {
+      if (!wake.wait_for(lk, std::chrono::seconds(5), [&] { return open && round != seen; })) {
+        --alive;
+        return;
+      }
+      seen = round;
+      ++joined;
+      lk.unlock();
+      work();
+      lk.lock();
+      if (--joined == 0) done.notify_all();
+    }
+  }
+  void run(size_t count, void (*c)(void *, size_t), void *x) {
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      n = count;
+      call = c;
+      ctx = x;
+      next = 0;
+      open = true;
+      ++round;
+      for (; alive < std::min<size_t>(helper_count(), count - 1); ++alive) {
+        try {
+          std::thread([this] { helper(); }).detach();
+        } catch (...) {  // no further thread: the loop runs on those there are
+          break;
+        }
+      }
+    }
+    wake.notify_all();
+    work();
+    std::unique_lock<std::mutex> lk(mu);
+    open = false;
+    done.wait(lk, [&] { return joined == 0; });
+  }
+};
+
+Helpers &helpers() {
+  // never destroyed: idle helpers may outlive static destruction; a forked child has none of its
+  // parent's threads and starts with its own
+  static std::atomic<Helpers *> current{nullptr};
+  Helpers *h = current.load();
+  if (!h || h->process != (long)getpid()) {
+    Helpers *fresh = new Helpers;
+    if (current.compare_exchange_strong(h, fresh)) h = fresh;
+    else delete fresh;
+  }
+  return *h;
+}
+
+}  // namespace
+
+void run_on_helpers(size_t n, void (*call)(void *, size_t), void *ctx) {
+  if (n == 0) return;
+  if (n == 1 || helper_count() == 0) {
+    for (size_t i = 0; i < n; ++i) call(ctx, i);
+    return;
+  }
+  Helpers &h = helpers();
+  if (!h.running.exchange(true)) {
+    h.run(n, call, ctx);
+    h.running = false;
+    return;
+  }
+  std::atomic<size_t> next{0};
+  auto work = [&]() {
+    for (size_t i = next.fetch_add(1); i < n; i = next.fetch_add(1)) call(ctx, i);
+  };
+  std::vector<std::thread> pool;
+  for (size_t t = 0; t < std::min<size_t>(helper_count(), n - 1); ++t) {
+    try {
+      pool.emplace_back(work);
+    } catch (...) {
+      break;
+    }
+  }
+  work();
+  for (auto &th : pool) th.join();
+}
 
 // ---------------------------------------------------------------- 4x4 algebra
 
