@@ -1,4 +1,4 @@
-// Element types and inner products of the CUDA-core triple products (sm_103a).
+// Element types and inner products of the triple products on the CUDA cores (sm_103a).
 //
 // FP64 products in fixed point.  The FP64 pipe of this GPU issues 2 multiply-adds per
 // SM and clock (measured; FP64 mma.sync 1.75), the integer pipe 63 32 x 32 + 64 bit
@@ -38,10 +38,6 @@ template <>
 struct Arith<true> {
   using Elem = int2;
   using Out = double;
-  struct Acc {  // sum hi hi', sum (hi lo' + lo hi')
-    long long hh, cr;
-  };
-  __device__ static int2 one() { return make_int2(1 << 27, 0); }  // 1.0 under exponent 1023
   static constexpr int VK = 2;  // elements per 128-bit shared load
   static constexpr int PAD = 2;  // row pitch TS + PAD
 };
@@ -50,8 +46,6 @@ template <>
 struct Arith<false> {
   using Elem = float;
   using Out = float;
-  using Acc = float;
-  __device__ static float one() { return 1.f; }
   static constexpr int VK = 4;
   static constexpr int PAD = 4;
 };
@@ -167,37 +161,7 @@ __device__ __forceinline__ void mm(const float *A, const float *B, int kc, int n
   }
 }
 
-// acc[a][b] += sum_k A[4a][k] B[8b][k] for a < NA and b < NB; row pitches pa and pb.  The loop
-// has no branches: one on a would be turned into selects of the 64-bit sums.
-template <int NA, int NB, int NAT, int NBT>
-__device__ __forceinline__ void mm_acc(const int2 *A, int pa, const int2 *B, int pb, int kc,
-                                       Arith<true>::Acc (&acc)[NAT][NBT]) {
-  pa *= 4;
-  pb *= 8;
-#pragma unroll 1
-  for (int k = 0; k < kc; k += 2, A += 2, B += 2) {
-    int4 y[NB];
-#pragma unroll
-    for (int b = 0; b < NB; ++b) y[b] = *reinterpret_cast<const int4 *>(B + b * pb);
-#pragma unroll
-    for (int a = 0; a < NA; ++a) {
-      const int4 x = *reinterpret_cast<const int4 *>(A + a * pa);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) mad(acc[a][b].hh, x.x, y[b].x);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) mad(acc[a][b].cr, x.x, y[b].y);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) mad(acc[a][b].hh, x.z, y[b].z);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) mad(acc[a][b].cr, x.y, y[b].x);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) mad(acc[a][b].cr, x.z, y[b].w);
-#pragma unroll
-      for (int b = 0; b < NB; ++b) mad(acc[a][b].cr, x.w, y[b].z);
-    }
-  }
-}
-
+// acc[a][b] += sum_k A[4a][k] B[8b][k] for a < NA and b < NB; row pitches pa and pb
 template <int NA, int NB, int NAT, int NBT>
 __device__ __forceinline__ void mm_acc(const float *A, int pa, const float *B, int pb, int kc,
                                        float (&acc)[NAT][NBT]) {
@@ -223,21 +187,18 @@ __device__ __forceinline__ void mm_acc(const float *A, int pa, const float *B, i
   }
 }
 
-// for the na <= NAT row groups and nb <= NBT column groups that hold outputs
-template <int NB, typename Elem, typename Acc, int NAT, int NBT>
-__device__ __forceinline__ void mm_rows(const Elem *A, int pa, const Elem *B, int pb, int kc, int na,
-                                        Acc (&acc)[NAT][NBT]) {
-  constexpr int T = NAT;
+// for the na <= 4 row groups and nb <= NBT column groups that hold outputs
+template <int NB, int NBT>
+__device__ __forceinline__ void mm_rows(const float *A, int pa, const float *B, int pb, int kc, int na,
+                                        float (&acc)[4][NBT]) {
   if (na == 1) mm_acc<1, NB>(A, pa, B, pb, kc, acc);
   else if (na == 2) mm_acc<2, NB>(A, pa, B, pb, kc, acc);
   else if (na == 3) mm_acc<3, NB>(A, pa, B, pb, kc, acc);
-  else if (T == 4 || na == 4) mm_acc<4, NB>(A, pa, B, pb, kc, acc);
-  else if (na <= 6) mm_acc<(T > 4 ? 6 : 4), NB>(A, pa, B, pb, kc, acc);
-  else mm_acc<T, NB>(A, pa, B, pb, kc, acc);
+  else mm_acc<4, NB>(A, pa, B, pb, kc, acc);
 }
-template <typename Elem, typename Acc, int NAT, int NBT>
-__device__ __forceinline__ void mm_any(const Elem *A, int pa, const Elem *B, int pb, int kc, int na, int nb,
-                                       Acc (&acc)[NAT][NBT]) {
+template <int NBT>
+__device__ __forceinline__ void mm_any(const float *A, int pa, const float *B, int pb, int kc, int na, int nb,
+                                       float (&acc)[4][NBT]) {
   if constexpr (NBT == 2) {
     if (nb == 1) mm_rows<1>(A, pa, B, pb, kc, na, acc);
     else mm_rows<2>(A, pa, B, pb, kc, na, acc);
@@ -249,15 +210,6 @@ __device__ __forceinline__ void mm_any(const Elem *A, int pa, const Elem *B, int
   }
 }
 
-__device__ __forceinline__ long long fold(const Arith<true>::Acc &x, int s) {
-  return (x.hh << s) + ((x.cr + (1ll << (28 - s))) >> (29 - s));
-}
-// between chunks of the inner dimension: the cross sum goes back below 2^29
-__device__ __forceinline__ void carry(Arith<true>::Acc &x) {
-  x.hh += x.cr >> 29;
-  x.cr &= (1ll << 29) - 1;
-}
-__device__ __forceinline__ void carry(float &) {}
 __device__ __forceinline__ unsigned magnitude(long long t) { return (unsigned)((t ^ (t >> 63)) >> 32); }
 
 // f 2^e for an f whose exponent is moderate (|e| stays below 1000, see tile_special)

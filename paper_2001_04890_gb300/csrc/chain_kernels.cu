@@ -675,9 +675,8 @@ cudaError_t launch_chain_f32ops(const ChainEntry *e, const ChainGroup *g, const 
 
 // The work items of a group: its kernel class (index into the counts) and columns.
 int chain_item_class(int m, int q, int nmax, int pmax) {
-  // class 0: what the kernel for small blocks holds in its tiles, at the larger of the two types'
-  // row pitches (limbs': pad2, floats': pad4 of chain_pipe.cu)
-  const int pitch = std::max(((nmax + 1) >> 2 << 2) + 2, ((nmax + 3) >> 3 << 3) + 4);
+  // class 0: what the FP32 kernel for small blocks (chain_pipe.cu) holds in its tiles, at its row pitch
+  const int pitch = ((nmax + 3) >> 3 << 3) + 4;
   if (m <= 16 && q <= 16 && nmax <= 32 && pmax <= 16 && std::max(m, pmax) * pitch <= kPipeTile) return 0;
   if (q <= 32) return m <= 16 ? 1 : 2;
   return q <= 64 ? 3 : q <= 96 ? 4 : 5;

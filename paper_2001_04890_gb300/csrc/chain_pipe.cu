@@ -1,14 +1,12 @@
-// H.psi on the CUDA cores (sm_103a): D = sum_e f_e X_e Y_e Z_e over prepared operands
-// (Sec. 2.2.1, Eq. dgemm: X = A_l, Y = psi^s, Z = A_r^T).
+// Prepared operands of H.psi, D = sum_e f_e X_e Y_e Z_e (Sec. 2.2.1, Eq. dgemm: X = A_l,
+// Y = psi^s, Z = A_r^T), and its FP32 products on the CUDA cores (sm_103a).
 //
 // The operators of a position are read by thousands of tasks each, the psi blocks by
 // hundreds, so both are put into the form that the inner loops take before the tasks run:
-// the operators once per position, psi once per call.  FP64 becomes 58-bit block-scaled
-// integers in two limbs (chain_arith.cuh has the arithmetic and its error), 8 bytes an
-// element like the double it stands for, with one exponent per block; the FP32 mode rounds
-// psi to FP32.
+// the operators once per position, psi once per call.  FP64 becomes digits under one exponent
+// per block (chain_digits.cuh, chain_mma.cu); the FP32 mode rounds psi to FP32.
 //
-// An image of a block is a ready-made run of shared-memory tiles: the summed index cut into
+// An FP32 image of a block is a ready-made run of shared-memory tiles: the summed index cut into
 // chunks of 32, each chunk rows x pitch with the summed index contiguous, zeros to the pitch.
 // The pitch is 4 banks mod 8, so that the 128-bit loads of a warp (8 rows) are free of
 // conflicts; any range of rows of a chunk is one contiguous copy.  A block has two images, of
@@ -19,6 +17,7 @@
 #include <climits>
 
 #include "chain_arith.cuh"
+#include "chain_digits.cuh"
 #include "kernels.cuh"
 
 namespace dmrg {
@@ -28,37 +27,42 @@ namespace {
 constexpr int KD = 32;  // depth of a chunk
 
 // row pitch of a chunk of w columns (elements)
-template <bool FX>
-__host__ __device__ constexpr int pitch_of(int w) {
-  return FX ? ((w + 1) >> 2 << 2) + 2 : ((w + 3) >> 3 << 3) + 4;
-}
-// elements of an image with R rows and K columns
+__host__ __device__ constexpr int pitch_of(int w) { return ((w + 3) >> 3 << 3) + 4; }
+// elements of an image with R rows and K columns (FX: of 8 bytes)
 template <bool FX>
 __host__ __device__ constexpr int64_t image_size(int R, int K) {
-  return (int64_t)R * ((K / KD) * pitch_of<FX>(KD) + (K % KD ? pitch_of<FX>(K % KD) : 0));
+  return FX ? dig_image_size(R, K) : (int64_t)R * ((K / KD) * pitch_of(KD) + (K % KD ? pitch_of(K % KD) : 0));
 }
 
 // ---------------------------------------------------------------- preparation of operands
 
-template <bool FX, typename T>
-__device__ __forceinline__ typename Arith<FX>::Elem convert(T x, int E) {
-  if constexpr (FX) return to_limbs((double)x, E);
-  else return (float)x;
-}
+template <bool FX>
+using ImageElem = typename Arith<FX>::Elem;  // 8 bytes, or a float
 
-// The image of the R x K view src(r, k) = src[r rs + k cs] by nthr threads.
-template <bool FX, typename T>
-__device__ __forceinline__ void write_image(typename Arith<FX>::Elem *dst, const T *src, int R, int K, int64_t rs,
-                                            int64_t cs, int E, int tid, int nthr) {
-  using Elem = typename Arith<FX>::Elem;
-  for (int k0 = 0; k0 < K; k0 += KD) {
-    const int w = min(KD, K - k0), P = pitch_of<FX>(w);
-    for (int t = tid; t < R * P; t += nthr) {
-      const int r = t / P, k = t - r * P;
-      dst[t] = k < w ? convert<FX>(src[r * rs + (k0 + k) * cs], E) : Elem();
+// The image of an R x K block whose element (r, k) is get(r, k), an integer or a float, by nthr threads.
+template <bool FX, bool OPERATOR, class Get>
+__device__ __forceinline__ void write_image(ImageElem<FX> *dst, int R, int K, int tid, int nthr, Get get) {
+  if constexpr (FX) {
+    write_digits<OPERATOR>(dst, R, K, tid, nthr, get);
+  } else {
+    for (int k0 = 0; k0 < K; k0 += KD) {
+      const int w = min(KD, K - k0), P = pitch_of(w);
+      for (int t = tid; t < R * P; t += nthr) {
+        const int r = t / P, k = t - r * P;
+        dst[t] = k < w ? get(r, k0 + k) : 0.f;
+      }
+      dst += (int64_t)R * P;
     }
-    dst += (int64_t)R * P;
   }
+}
+// and of the view src[r rs + k cs]
+template <bool FX, bool OPERATOR, typename T>
+__device__ __forceinline__ void write_view(ImageElem<FX> *dst, const T *src, int R, int K, int64_t rs, int64_t cs, int E,
+                                           int tid, int nthr) {
+  write_image<FX, OPERATOR>(dst, R, K, tid, nthr, [&](int r, int k) {
+    if constexpr (FX) return to_fixed((double)src[r * rs + k * cs], E);
+    else return (float)src[r * rs + k * cs];
+  });
 }
 
 template <bool FX, typename T>
@@ -86,19 +90,18 @@ __global__ void __launch_bounds__(256) op_images_kernel(const OpSlab *__restrict
     const int64_t i = b - s.first, size = (int64_t)s.rows * s.cols;
     Elem *img = reinterpret_cast<Elem *>(s.img) + i * (image_size<FX>(s.rows, s.cols) + image_size<FX>(s.cols, s.rows));
     if (s.src == ~0ull) {  // an identity: its own transpose
-      for (int k0 = 0; k0 < s.cols; k0 += KD) {
-        const int w = min(KD, s.cols - k0), P = pitch_of<FX>(w);
-        for (int t = lane; t < s.rows * P; t += 32) img[t] = t / P == k0 + t % P ? Arith<FX>::one() : Elem();
-        img += s.rows * P;
-      }
+      write_image<FX, true>(img, s.rows, s.cols, lane, 32, [](int r, int k) {
+        if constexpr (FX) return r == k ? 1ll << 57 : 0ll;
+        else return r == k ? 1.f : 0.f;
+      });
       if (lane == 0) exps[b] = 1023;
       continue;
     }
     const T *src = reinterpret_cast<const T *>(s.src * sizeof(T)) + i * size;
     const int E = block_exponent<FX>(src, size, lane);
     if (E >= 0) {
-      write_image<FX>(img, src, s.rows, s.cols, s.cols, 1, E, lane, 32);
-      write_image<FX>(img + image_size<FX>(s.rows, s.cols), src, s.cols, s.rows, 1, s.cols, E, lane, 32);
+      write_view<FX, true>(img, src, s.rows, s.cols, s.cols, 1, E, lane, 32);
+      write_view<FX, true>(img + image_size<FX>(s.rows, s.cols), src, s.cols, s.rows, 1, s.cols, E, lane, 32);
     }
     if (lane == 0) exps[b] = (int16_t)E;
   }
@@ -130,12 +133,12 @@ __global__ void __launch_bounds__(128) psi_images_kernel(const PsiSpan *__restri
     if (tid == 0) exps[blockIdx.x] = E;
     if (E < 0) return;
   }
-  write_image<FX>(out + s.img, src, s.rows, s.cols, s.cols, 1, E, tid, 128);
-  write_image<FX>(out + s.img + image_size<FX>(s.rows, s.cols), src, s.cols, s.rows, 1, s.cols, E, tid, 128);
+  write_view<FX, false>(out + s.img, src, s.rows, s.cols, s.cols, 1, E, tid, 128);
+  write_view<FX, false>(out + s.img + image_size<FX>(s.rows, s.cols), src, s.cols, s.rows, 1, s.cols, E, tid, 128);
 }
 
 // The tasks of one chunk in the kernel's order and cut into stacks of consecutive tasks that
-// share a psi block.  Limbs: sorted by psi block (kSortSpan at a time), so that those are many;
+// share a psi block.  Digits: sorted by psi block (kSortSpan at a time), so that those are many;
 // FP32 tasks stay in the list's order, in which their FP32 sum is formed.
 constexpr int kSortSpan = 1024;
 
@@ -164,10 +167,7 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
           const int mid = (lo + hi + 1) >> 1;
           if (B[mid].off <= y) lo = mid; else hi = mid - 1;
         }
-        // limbs: tasks with a coefficient other than +-2^k run alone
-        const double f = E[g.first + b0 + i].f;
-        const bool alone = FX && ((__double2hiint(f) & 0xfffff) != 0 || __double2loint(f) != 0);
-        k = (unsigned long long)(2 * lo + (alone ? 1 : 0)) << 32 | (unsigned)i;
+        k = (unsigned long long)lo << 32 | (unsigned)i;
       }
       key[i] = k;
     }
@@ -210,8 +210,7 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
       bool head = false;
       PipeStack st{};
       if (i < cnt) {
-        const int yb = (int)(key[i] >> 33);
-        const bool alone = (key[i] >> 32) & 1;
+        const int yb = (int)(key[i] >> 32);
         const ChainEntry e = E[g.first + b0 + (int)(unsigned)key[i]];
         const bool xt = e.xcs != 1 || (e.xrs == 1 && e.n > 1), yt = e.ycs != 1 || (e.yrs == 1 && e.p > 1),
                    zt = e.zcs != 1 || (e.zrs == 1 && g.q > 1);
@@ -256,7 +255,7 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
         if (FX && (ef > 1023 + 100 || ef < 1023 - 100)) ex = -1;  // a coefficient that needs FP64
         p.w = FX ? (ex < 0 || ez < 0 ? INT_MIN : ex + ez + ef) : 0;
         p.src = g.first + b0 + (int)(unsigned)key[i];
-        const int cap = alone ? 1 : pipe_stack_cap(FX, g.tile0, g.m, g.q, e.n, e.p);
+        const int cap = pipe_stack_cap(FX, g.tile0, g.m, g.q, e.n, e.p);
         head = (i - run0[i]) % cap == 0;
         st.e = g.first + b0 + i;
         st.ns = min(cap, run1[i] - i + 1);
@@ -299,7 +298,7 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
   }
 }
 
-// ---------------------------------------------------------------- the kernel
+// ---------------------------------------------------------------- the FP32 kernel
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
@@ -318,121 +317,52 @@ __device__ __forceinline__ void copy_run(void *dst, const void *src, int n, int 
     cp_async16(static_cast<char *>(dst) + o, static_cast<const char *>(src) + o);
 }
 
-// Barrier of the group of threads [id nthr, (id + 1) nthr) of the CTA (whole warps).
-__device__ __forceinline__ void group_sync(int id, int nthr) {
-  if (nthr == 32)
-    __syncwarp();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "r"(nthr) : "memory");
-}
-
-// Group shapes.  A warp has 16 rows.  SMALL: output blocks of at most 16 x 16 and tasks whose X,
+// CTA shapes.  A warp has 16 rows.  SMALL: output blocks of at most 16 x 16 and tasks whose X,
 // Y and Z fit kPipeTile, 16 columns a warp; else 32 columns.
-//
-// Threads an SM holds of the kernel for small blocks.  At 512 a lane's 128 registers do not hold
-// the limb sums, two stacks' descriptions and the addresses; measured at 384 / 512: H psi, 8
-// orbitals, M 64: 196 / 216 us; 16 vectors, 24 orbitals, M 512: 13.4 / 12.8 ms; Davidson, 10
-// orbitals, M 128: 157 / 168 ms.
-constexpr int kSmallThreads = 384;
-template <bool FX, bool SMALL, int WC>
+template <bool SMALL, int WC>
 struct PipeShape {
   static constexpr int NA = 4;              // rows per lane
   static constexpr int NB = SMALL ? 2 : 4;  // columns per lane
   static constexpr int CW = 8 * NB;         // columns of a warp
-  static constexpr int PI = pitch_of<FX>(KD);  // row pitch of a whole chunk
-  static constexpr int MAXTHREADS = WC == 1 ? 128 : 64 * WC;
-  static constexpr int MINB = (SMALL ? kSmallThreads : WC == 4 ? 256 : 384) / MAXTHREADS;
+  static constexpr int PI = pitch_of(KD);   // row pitch of a whole chunk
+  static constexpr int MAXTHREADS = 64 * WC;
+  static constexpr int MINB = (WC == 4 ? 256 : 384) / MAXTHREADS;
 };
 
-// Shared memory of a group (elements): the X tile, each of the two Y / Z buffers, and the T tiles
-// with row pitch pt, sized for the largest dimensions of the launch's tasks.
+// Shared memory (elements): the X tile, each of the two Y / Z buffers, and the T tiles with row
+// pitch pt, sized for the largest dimensions of the launch's tasks.
 struct PipeSmem {
-  int x, b, pt, group;
+  int x, b, pt, total;
 };
-
-// The stacks of an item that fixed point does not take, in FP64 from the operators; added to
-// the item's output, which the kernel has written.
-__device__ __noinline__ void slow_stacks(const PipeEntry *P, const PipeStack *S, int nst, const ChainEntry *E,
-                                         const int *pexp, const double *psi, const ChainGroup *gp, int r0, int c0,
-                                         int rows, int cols, uint64_t db, double *T) {
-  const ChainGroup g = *gp;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  double *D = reinterpret_cast<double *>(db + g.d * 8ull);
-  for (int st = 0; st < nst; ++st) {
-    if (!S[st].flags && pexp[S[st].yb] >= 0) continue;
-    for (int i = S[st].e; i < S[st].e + S[st].ns; ++i) {
-      const ChainEntry e = E[P[i].src];
-      const bool xi = e.x == ~0ull, zi = e.z == ~0ull;
-      const double *X = reinterpret_cast<const double *>(e.x * 8ull), *Y = psi + e.y;
-      const double *Z = reinterpret_cast<const double *>(e.z * 8ull);
-      for (int p0 = 0; p0 < e.p; p0 += 16) {
-        const int pc = min(16, e.p - p0);
-        __syncthreads();
-        for (int t = tid; t < rows * pc; t += nthr) {
-          const int64_t r = r0 + t / pc, k = p0 + t % pc;
-          double s = 0.0;
-          if (xi) s = Y[r * e.yrs + k * e.ycs];
-          else
-            for (int64_t j = 0; j < e.n; ++j) s = fma(X[r * e.xrs + j * e.xcs], Y[j * e.yrs + k * e.ycs], s);
-          T[(t / pc) * 16 + t % pc] = s;
-        }
-        __syncthreads();
-        for (int t = tid; t < rows * cols; t += nthr) {
-          const int64_t r = t / cols, c = c0 + t % cols;
-          double s = 0.0;
-          if (zi) {
-            if (c < p0 || c >= p0 + pc) continue;
-            s = T[r * 16 + c - p0];
-          } else {
-            for (int64_t k = 0; k < pc; ++k) s = fma(T[r * 16 + k], Z[(p0 + k) * e.zrs + c * e.zcs], s);
-          }
-          double *d = D + (r0 + r) * g.drs + c * g.dcs;
-          *d = fma(e.f, s, *d);
-        }
-      }
-    }
-  }
-}
 
 // One work item per CTA: rows [r0, r0 + 16 wr) and columns [c0, c0 + CW WC) of one chunk's
-// output block.  The CTA holds one group of wr x WC warps, or (WC = 1) several that take the
-// chunk's stacks in turn and whose sums are added in group order.  Lane (i, j) of a warp's
-// 4 x 8 lane grid has rows i + 4 a and columns j + 8 b of the warp's tile, so a ragged block
-// wastes at most 3 rows and 7 columns.
+// output block, wr x WC warps.  Lane (i, j) of a warp's 4 x 8 lane grid has rows i + 4 a and
+// columns j + 8 b of the warp's tile, so a ragged block wastes at most 3 rows and 7 columns.
 //
-// A group works through units: for every stack and every CW WC columns of T, the chunks of
+// The CTA works through units: for every stack and every CW WC columns of T, the chunks of
 // stage 1 (T = X Y) and then those of stage 2 (D += f T Z).  A unit's tiles are copied while
 // the unit before it is computed: X to its own buffer, Y and Z to two buffers in turn.
 //
 // The X of a stack's tasks lie below one another in the X tile, so stage 1 is one product with
-// the Y that they share; their parts of T lie beside one another, and stage 2 sums over them.
-// For that the parts of T get one scale, coefficients +-2^k and all; a task with another
-// coefficient (a one-site term) is a stack of its own.
-template <bool FX, bool SMALL, int WC>
-__global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShape<FX, SMALL, WC>::MINB)
+// the Y that they share; their parts of T lie beside one another, and stage 2 adds their
+// products to D task by task: the FP32 sums are formed in the task list's order, whatever the
+// shapes and stacks.
+template <bool SMALL, int WC>
+__global__ void __launch_bounds__(PipeShape<SMALL, WC>::MAXTHREADS, PipeShape<SMALL, WC>::MINB)
     chain_pipe_kernel(const PipeEntry *__restrict__ E, const PipeStack *__restrict__ stacks,
-                      const int *__restrict__ nstacks, const ChainEntry *__restrict__ tasks,
-                      const ChainGroup *__restrict__ G, const ChainItem *__restrict__ items, int wr, PipeSmem sm,
-                      const typename Arith<FX>::Elem *__restrict__ psi, const int *__restrict__ pexp,
-                      const double *__restrict__ psi64, uint64_t db) {
-  using A = Arith<FX>;
-  using Elem = typename A::Elem;
-  using Out = typename A::Out;
-  using Acc = typename A::Acc;
-  using S = PipeShape<FX, SMALL, WC>;
-  constexpr int NA = S::NA, NB = S::NB, CW = S::CW, PI = S::PI, VK = A::VK, ES = (int)sizeof(Elem);
+                      const int *__restrict__ nstacks, const ChainGroup *__restrict__ G,
+                      const ChainItem *__restrict__ items, int wr, PipeSmem sm, const float *__restrict__ psi,
+                      uint64_t db) {
+  using S = PipeShape<SMALL, WC>;
+  constexpr int NA = S::NA, NB = S::NB, CW = S::CW, PI = S::PI, VK = 4, ES = (int)sizeof(float);
   extern __shared__ __align__(16) unsigned char pipe_smem[];
-  __shared__ int te[8][WC];   // exponents of the T tiles
-  const int gthr = 32 * wr * WC;
-  const int grp = WC == 1 ? (int)threadIdx.x / gthr : 0, ngrp = WC == 1 ? (int)blockDim.x / gthr : 1;
-  const int tid = (int)threadIdx.x - grp * gthr, warp = tid >> 5, lane = tid & 31;
+  const int nthr = 32 * wr * WC, tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wrow = warp / WC, wcol = warp % WC;
   const int lr = lane >> 3, lc = lane & 7;
   const int PT = sm.pt;
-  Elem *Xs = reinterpret_cast<Elem *>(pipe_smem) + grp * sm.group;
-  Elem *Bs = Xs + sm.x;
-  Elem *Ts = Bs + 2 * sm.b + wrow * WC * 16 * PT;  // this warp row's tiles
-  int *tex = WC > 1 ? te[wrow] : te[threadIdx.x >> 5];
+  float *Xs = reinterpret_cast<float *>(pipe_smem);
+  float *Bs = Xs + sm.x;
+  float *Ts = Bs + 2 * sm.b + wrow * WC * 16 * PT;  // this warp row's tiles
   const ChainItem it = items[blockIdx.x];
   const ChainGroup *gp = G + it.g;
   const int gm = gp->m, gq = gp->q, gfirst = gp->first;
@@ -442,54 +372,44 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
   const int rw = WC == 1 && wr == 1 ? 16 : (mi + 4 * wr - 1) / (4 * wr) * 4;  // rows of a warp
   const int m = min(rw, mi - rw * wrow);                                     // of this warp
   const int q = min(CW, qi - CW * wcol);
-  Out D[4][NB];
+  float D[4][NB];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < NB; ++b) D[a][b] = 0;
-  bool any_special = false;
-  // FP32 sums over the inner dimension keep one order: chunks of 32 added up for blocks of at
+    for (int b = 0; b < NB; ++b) D[a][b] = 0.f;
+  // sums over the inner dimension keep one order: chunks of 32 added up for blocks of at
   // most 32 x 32, running on for larger ones
-  const bool apart = !FX && gm <= 32 && gq <= 32;
+  const bool apart = gm <= 32 && gq <= 32;
 
-  // A stack (PipeStack as read, and the exponent of its Y).  It is read one stack ahead, and
-  // what it points to is asked for in time, so that no copy waits for a chain of loads.
+  auto sync = [&]() {
+    if (nthr == 32) __syncwarp();
+    else __syncthreads();
+  };
+  // A stack (PipeStack as read).  It is read one stack ahead, and what it points to is asked for in
+  // time, so that no copy waits for a chain of loads.
   struct Stack {
     int4 d;
-    int ey;
     __device__ __forceinline__ int e() const { return d.x; }
     __device__ __forceinline__ int n() const { return d.y & 0xffff; }
     __device__ __forceinline__ int p() const { return (int)((unsigned)d.y >> 16); }
     __device__ __forceinline__ uint32_t y() const { return (uint32_t)d.z; }
-    __device__ __forceinline__ int yb() const { return d.w & 0xffffff; }
     __device__ __forceinline__ int ns() const { return (d.w >> 24) & 15; }
-    __device__ __forceinline__ bool special() const { return (unsigned)d.w >> 28 || ey < 0; }
   };
-  int si = grp;
+  int si = 0;
   auto member = [&](int ns) { return ns <= 1 ? 0 : tid >> (5 - (32 - __clz(ns - 1))); };  // stacks: one warp
-  auto take = [&](Stack &t) {  // ns() = 0: no further stack of this group
+  auto take = [&](Stack &t) {  // ns() = 0: no further stack
     t.d = si < nst ? *reinterpret_cast<const int4 *>(stk + si) : make_int4(0, 0, 0, 0);
-    t.ey = 0;
-    si += ngrp;
+    ++si;
   };
-  auto ask = [&](Stack &t) {  // for the exponent of Y and this thread's share of the entries
-    if (t.ns() == 0) return;
-    if (FX) t.ey = pexp[t.yb()];
-    prefetch(E + t.e() + min(member(t.ns()), t.ns() - 1));
-  };
-  auto skip_special = [&](Stack &t) {
-    while (FX && t.ns() > 0 && t.special()) {
-      any_special = true;
-      take(t);
-      ask(t);
-    }
+  auto ask = [&](const Stack &t) {  // for this thread's share of the entries
+    if (t.ns() > 0) prefetch(E + t.e() + min(member(t.ns()), t.ns() - 1));
   };
   // Copy the tiles of a unit of t: chunk c of stage 1 or (two) of stage 2, columns of T from p0.
-  auto copy_unit = [&](const Stack &t, int p0, int c, bool two, Elem *B) {
-    const int ns = t.ns(), lg = ns <= 1 ? 0 : 32 - __clz(ns - 1), mem = lg ? tid >> (5 - lg) : 0, sub = gthr >> lg,
+  auto copy_unit = [&](const Stack &t, int p0, int c, bool two, float *B) {
+    const int ns = t.ns(), lg = ns <= 1 ? 0 : 32 - __clz(ns - 1), mem = lg ? tid >> (5 - lg) : 0, sub = nthr >> lg,
               st = lg ? tid & (sub - 1) : tid;
     const int k0 = two ? p0 + c * CW : c * KD;  // summed index
-    const int w = min(KD, (two ? t.p() : t.n()) - k0), P = pitch_of<FX>(w);
+    const int w = min(KD, (two ? t.p() : t.n()) - k0), P = pitch_of(w);
     const int R = two ? gq : gm, r0 = two ? it.c0 : it.r0, rows = two ? qi : mi;
     if (mem < ns) {
       const PipeEntry &e = E[t.e() + mem];
@@ -498,14 +418,13 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
                st, sub);
     }
     if (!two)
-      copy_run(B, psi + t.y() + (int64_t)(k0 / KD) * t.p() * PI + p0 * P, min(CW * WC, t.p() - p0) * P * ES, tid, gthr);
+      copy_run(B, psi + t.y() + (int64_t)(k0 / KD) * t.p() * PI + p0 * P, min(CW * WC, t.p() - p0) * P * ES, tid, nthr);
     cp_commit();
   };
 
   Stack u, nx;  // the stack at hand and the next one
   take(u);
   ask(u);
-  skip_special(u);
   if (u.ns() > 0) {
     copy_unit(u, 0, 0, false, Bs);
     take(nx);
@@ -513,7 +432,7 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
   int p0 = 0, c = 0;
   bool two = false;
   int par_b = 0;  // buffer of the current unit
-  Acc acc[NA][NB];
+  float acc[NA][NB];
 #pragma unroll 1
   while (u.ns() > 0) {
     const int nch = (u.n() + KD - 1) / KD;
@@ -535,133 +454,65 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
       }
     }
     cp_wait<0>();
-    group_sync(grp, gthr);  // the tiles are here, the unit before this one has been computed
+    sync();  // the tiles are here, the unit before this one has been computed
     const bool late = !over && !two && !vtwo;  // X is still in use: copied after this unit
     if (!two && c == 0 && p0 == 0) ask(nx);
     if (over) {
-      skip_special(nx);
       if (nx.ns() > 0) copy_unit(nx, 0, 0, false, Bs + (par_b ^ 1) * sm.b);
     } else if (!late) {
       copy_unit(u, vp, vc, vtwo, Bs + (par_b ^ 1) * sm.b);
     }
-    const Elem *B = Bs + par_b * sm.b;
+    const float *B = Bs + par_b * sm.b;
     const int ns = u.ns();
     const int pc = min(CW, u.p() - p0 - CW * (two ? c : wcol));  // columns of the T tile at hand
     const int pt = (pc + VK - 1) / VK * VK;                          // a member's columns in the tile
     const bool busy = m > 0 && (two ? q : pc) > 0;
     const int rows = two ? m : ns * m, na = (rows + 3) >> 2, nb = ((two ? q : pc) + 7) >> 3;
     if (busy) {
-      // ---- sums of the unit: X Y, or over the members of T Z
-      const int kc = two ? pc : min(KD, u.n() - c * KD), P = pitch_of<FX>(kc);
+      // ---- sums of the unit: X Y, or member by member T Z
+      const int kc = two ? pc : min(KD, u.n() - c * KD), P = pitch_of(kc);
       if (two || c == 0 || apart) {
 #pragma unroll
         for (int a = 0; a < NA; ++a)
 #pragma unroll
-          for (int b = 0; b < NB; ++b) acc[a][b] = Acc{};
-      } else {
-#pragma unroll
-        for (int a = 0; a < NA; ++a)
-#pragma unroll
-          for (int b = 0; b < NB; ++b) carry(acc[a][b]);
+          for (int b = 0; b < NB; ++b) acc[a][b] = 0.f;
       }
-      const Elem *Ar = two ? Ts + c * 16 * PT + lr * PT : Xs + (rw * wrow + lr) * P;
-      const Elem *Br = B + (wcol * CW + lc) * P;
+      const float *Ar = two ? Ts + c * 16 * PT + lr * PT : Xs + (rw * wrow + lr) * P;
+      const float *Br = B + (wcol * CW + lc) * P;
 #pragma unroll 1
       for (int mem = 0; mem < (two ? ns : 1); ++mem, Ar += pt, Br += qi * P) {
         mm_any(Ar, two ? PT : P, Br, P, kc, na, nb, acc);
-        if constexpr (!FX) {
-          if (two) {  // D += f (T Z), task by task
-            const float f = (float)E[u.e() + mem].f;
+        if (two) {  // D += f (T Z), task by task
+          const float f = (float)E[u.e() + mem].f;
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+          for (int a = 0; a < 4; ++a)
 #pragma unroll
-              for (int b = 0; b < NB; ++b) {
-                D[a][b] = fmaf(f, acc[a][b], D[a][b]);
-                acc[a][b] = 0.f;
-              }
-          }
+            for (int b = 0; b < NB; ++b) {
+              D[a][b] = fmaf(f, acc[a][b], D[a][b]);
+              acc[a][b] = 0.f;
+            }
         }
       }
     }
-    if (busy && two) {
-      if constexpr (FX) {  // D += 2^e (sums)
-        // a single task's coefficient is applied here; those of a stack are +-2^k and are in T
-        const double f1 = ns == 1 ? E[u.e()].f : 1.0;
-        const int e2 = 58 - 1 + (WC > 1 ? tex[c] : tex[0]);
-        const double sc = __hiloint2double((__double2hiint(f1) & 0x800fffff) | ((e2 + 1023) << 20), __double2loint(f1));
+    if (busy && !two && (apart || c == nch - 1)) {
+      float *T = Ts + wcol * 16 * PT + lc;
+      const float invm = 1.0f / (float)m;
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
-          if (a < na) {
+      for (int a = 0; a < NA; ++a) {
+        if (a < na) {
+          const int row = lr + 4 * a, mem = ns > 1 ? small_div(row, invm) : 0;
+          if (row < rows) {
+            float *Tr = T + (row - mem * m) * PT + mem * pt;
 #pragma unroll
             for (int b = 0; b < NB; ++b)
-              if (b < nb) D[a][b] = fma(sc, (double)fold(acc[a][b], 1), D[a][b]);
-          }
-      }
-    } else if (busy) {
-      if (apart || c == nch - 1) {
-        Elem *T = Ts + wcol * 16 * PT + lc;
-        const float invm = 1.0f / (float)m;
-        if constexpr (FX) {
-          // the members' weights below the largest one (bits 0-5) and signs (bit 8): their parts
-          // of T get one scale
-          const int w = lane < ns ? E[u.e() + lane].w : INT_MIN;
-          const int wmax = __reduce_max_sync(kFull, w);
-          int below = 0;
-          if (ns > 1 && lane < ns) below = min(wmax - w, 62) | (__double2hiint(E[u.e() + lane].f) < 0 ? 256 : 0);
-          unsigned mx = 0;
-#pragma unroll
-          for (int a = 0; a < NA; ++a)
-            if (a < na) {
-              const int row = lr + 4 * a, sh = ns > 1 ? __shfl_sync(kFull, below, small_div(row, invm)) & 63 : 0;
-#pragma unroll
-              for (int b = 0; b < NB; ++b) {
-                const unsigned h = sh < 32 ? magnitude(acc[a][b].hh) >> sh : 0u;
-                mx = max(mx, b < nb && lc + 8 * b < pc && row < rows ? h : 0u);
-              }
-            }
-          mx = __reduce_max_sync(kFull, mx);
-          const int up = __clz(mx | 1) - 7;  // T = hh 2^(up - sh) + cross, below 2^57
-          if (lane == 0) tex[WC > 1 ? wcol : 0] = wmax + u.ey - 2158 - 1023 - 1079 + 58 - up;
-          const bool down = ns > 1 || up < 0;
-#pragma unroll
-          for (int a = 0; a < NA; ++a) {
-            if (a < na) {
-              const int row = lr + 4 * a, mem = ns > 1 ? small_div(row, invm) : 0;
-              const int v = ns > 1 ? __shfl_sync(kFull, below, mem) : 0;
-              const int net = up - (v & 63), l = max(net, 0), r = max(-net, 0);
-              const long long half = 1ll << (28 - l), rhalf = (1ll << r) >> 1, sg = -(long long)(v >> 8);
-              Elem *Tr = T + (row - mem * m) * PT + mem * pt;
-              if (row < rows) {
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                  if (lc + 8 * b < pt) {
-                    long long t = (acc[a][b].hh << l) + ((acc[a][b].cr + half) >> (29 - l));
-                    if (down) t = (((t + rhalf) >> r) ^ sg) - sg;
-                    Tr[8 * b] = lc + 8 * b < pc ? limbs(t) : Elem();
-                  }
-                }
-              }
-            }
-          }
-        } else {
-#pragma unroll
-          for (int a = 0; a < NA; ++a) {
-            if (a < na) {
-              const int row = lr + 4 * a, mem = ns > 1 ? small_div(row, invm) : 0;
-              if (row < rows) {
-                Elem *Tr = T + (row - mem * m) * PT + mem * pt;
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-                  if (lc + 8 * b < pt)
-                    Tr[8 * b] = lc + 8 * b < pc ? (apart && c > 0 ? Tr[8 * b] + acc[a][b] : acc[a][b]) : 0.f;
-              }
-            }
+              if (lc + 8 * b < pt)
+                Tr[8 * b] = lc + 8 * b < pc ? (apart && c > 0 ? Tr[8 * b] + acc[a][b] : acc[a][b]) : 0.f;
           }
         }
       }
     }
     if (late) {
-      group_sync(grp, gthr);
+      sync();
       copy_unit(u, vp, vc, vtwo, Bs + (par_b ^ 1) * sm.b);
     }
     par_b ^= 1;
@@ -673,60 +524,22 @@ __global__ void __launch_bounds__(PipeShape<FX, SMALL, WC>::MAXTHREADS, PipeShap
       if (u.ns() > 0) take(nx);
     }
   }
-  if constexpr (WC == 1) {
-    if (ngrp > 1) {  // the groups' sums, added in group order
-      __syncthreads();
-      Out *mine = reinterpret_cast<Out *>(pipe_smem) + (size_t)threadIdx.x * (4 * NB + 1);
-      if (grp > 0) {
+  const int drs = gp->drs, dcs = gp->dcs;
+  double *Dout = reinterpret_cast<double *>(db + gp->d * 8ull) + (int64_t)(it.r0 + rw * wrow) * drs +
+                 (int64_t)(it.c0 + CW * wcol) * dcs;
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-          for (int b = 0; b < NB; ++b) mine[a * NB + b] = D[a][b];
-      }
-      __syncthreads();
-      if (grp == 0) {
-        for (int h = 1; h < ngrp; ++h) {
-          const Out *other = reinterpret_cast<const Out *>(pipe_smem) + (size_t)(h * gthr + tid) * (4 * NB + 1);
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < NB; ++b) D[a][b] += other[a * NB + b];
-        }
-      }
-    }
-  }
-  if (grp == 0) {
-    const int drs = gp->drs, dcs = gp->dcs;
-    double *Dout = reinterpret_cast<double *>(db + gp->d * 8ull) + (int64_t)(it.r0 + rw * wrow) * drs +
-                   (int64_t)(it.c0 + CW * wcol) * dcs;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < NB; ++b)
-        if (lr + 4 * a < m && lc + 8 * b < q)
-          Dout[(int64_t)(lr + 4 * a) * drs + (int64_t)(lc + 8 * b) * dcs] = (double)D[a][b];
-  }
-  if constexpr (FX) {
-    if (__syncthreads_or(any_special))
-      slow_stacks(E, stk, nst, tasks, pexp, psi64, gp, it.r0, it.c0, mi, qi, db, reinterpret_cast<double *>(pipe_smem));
-  }
+    for (int b = 0; b < NB; ++b)
+      if (lr + 4 * a < m && lc + 8 * b < q)
+        Dout[(int64_t)(lr + 4 * a) * drs + (int64_t)(lc + 8 * b) * dcs] = (double)D[a][b];
 }
 
-// Groups that share a chunk's tasks: chunks of many tasks are shared, so that no CTA runs on
-// when the others are done, and so are chunks that alone would not fill the GPU.
-int groups_per_item(int n, int64_t tasks, int wr, int resident) {
-  int k = 1;
-  while (32 * wr * k < 128 && ((long long)n * wr * k < resident || tasks > 16ll * k * n)) k *= 2;
-  return k;
-}
-
-template <bool FX, bool SMALL, int WC>
-cudaError_t launch_pipe(const PipeArgs &a, const ChainItem *items, const PipeClass &c, int wr, bool share,
-                        cudaStream_t s) {
+template <bool SMALL, int WC>
+cudaError_t launch_pipe(const PipeArgs &a, const ChainItem *items, const PipeClass &c, int wr, cudaStream_t s) {
   if (c.items <= 0) return cudaSuccess;
-  using S = PipeShape<FX, SMALL, WC>;
-  using Elem = typename Arith<FX>::Elem;
-  auto pitch = [](int w) { return pitch_of<FX>(w < KD ? w : KD); };
+  using S = PipeShape<SMALL, WC>;
+  auto pitch = [](int w) { return pitch_of(w < KD ? w : KD); };
   const int mx = SMALL ? 0 : std::min(c.m, 16 * wr), qx = std::min(c.q, S::CW * WC), px = std::min(c.p, S::CW * WC);
   PipeSmem sm;
   // stacks of the small classes fill tiles of fixed size (pipe_stack_cap)
@@ -734,21 +547,17 @@ cudaError_t launch_pipe(const PipeArgs &a, const ChainItem *items, const PipeCla
   sm.b = SMALL ? kPipeTile : std::max(px * pitch(c.n), (wr == 1 ? 32 : qx) * pitch(c.p));
   sm.pt = WC == 1 && c.p > 16 ? pitch(c.p) : pitch(KD);
   if (wr == 1) sm.pt = pitch(SMALL ? 16 : KD);
-  sm.group = sm.x + 2 * sm.b + wr * WC * 16 * sm.pt;
-  sm.group = std::max(sm.group, 32 * wr * WC * (4 * S::NB + 1));  // the exchange of the groups' sums
-  const int bytes = sm.group * (int)sizeof(Elem);
-  const int groups = share && FX ? groups_per_item(c.items, c.tasks, wr, (SMALL ? kSmallThreads / 32 : 12) * 152) : 1;
-  auto kern = chain_pipe_kernel<FX, SMALL, WC>;
+  sm.total = sm.x + 2 * sm.b + wr * WC * 16 * sm.pt;
+  auto kern = chain_pipe_kernel<SMALL, WC>;
   const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
   if (err != cudaSuccess) return err;
   add_kernel_launches(1);
-  kern<<<c.items, 32 * wr * WC * groups, groups * bytes, s>>>(a.e, a.stacks, a.nstacks, a.tasks, a.g, items, wr, sm,
-                                                             static_cast<const Elem *>(a.psi), a.pexp, a.psi64, a.db);
+  kern<<<c.items, 32 * wr * WC, sm.total * sizeof(float), s>>>(a.e, a.stacks, a.nstacks, a.g, items, wr, sm,
+                                                               static_cast<const float *>(a.psi), a.db);
   return cudaGetLastError();
 }
 
-template <bool FX>
-cudaError_t launch_pipe_all(const PipeArgs &a, const ChainItem *items, const PipeClass *c, bool wide, cudaStream_t s,
+cudaError_t launch_pipe_f32(const PipeArgs &a, const ChainItem *items, const PipeClass *c, cudaStream_t s,
                             cudaStream_t s1, cudaStream_t s2) {
   cudaError_t err;
   auto next = [&](int cls) {
@@ -757,20 +566,19 @@ cudaError_t launch_pipe_all(const PipeArgs &a, const ChainItem *items, const Pip
     return p;
   };
   const ChainItem *i5 = next(5), *i4 = next(4), *i3 = next(3), *i2 = next(2), *i1 = next(1), *i0 = next(0);
-  if ((err = launch_pipe<FX, false, 4>(a, i5, c[5], 2, false, s1)) != cudaSuccess) return err;
-  if ((err = launch_pipe<FX, false, 3>(a, i4, c[4], 2, false, s)) != cudaSuccess) return err;
-  if ((err = launch_pipe<FX, false, 2>(a, i3, c[3], 2, false, s1)) != cudaSuccess) return err;
-  if ((err = launch_pipe<FX, false, 1>(a, i2, c[2], 2, wide, s)) != cudaSuccess) return err;
-  if ((err = launch_pipe<FX, false, 1>(a, i1, c[1], 1, wide, s1)) != cudaSuccess) return err;
-  return launch_pipe<FX, true, 1>(a, i0, c[0], 1, wide, s2);
+  if ((err = launch_pipe<false, 4>(a, i5, c[5], 2, s1)) != cudaSuccess) return err;
+  if ((err = launch_pipe<false, 3>(a, i4, c[4], 2, s)) != cudaSuccess) return err;
+  if ((err = launch_pipe<false, 2>(a, i3, c[3], 2, s1)) != cudaSuccess) return err;
+  if ((err = launch_pipe<false, 1>(a, i2, c[2], 2, s)) != cudaSuccess) return err;
+  if ((err = launch_pipe<false, 1>(a, i1, c[1], 1, s1)) != cudaSuccess) return err;
+  return launch_pipe<true, 1>(a, i0, c[0], 1, s2);
 }
 
 }  // namespace
 
 cudaError_t launch_chain_pipe(const PipeArgs &a, bool f32, const ChainItem *items, const PipeClass *classes, int wide,
                               cudaStream_t s, cudaStream_t s1, cudaStream_t s2) {
-  return f32 ? launch_pipe_all<false>(a, items, classes, wide != 0, s, s1, s2)
-             : launch_pipe_all<true>(a, items, classes, wide != 0, s, s1, s2);
+  return f32 ? launch_pipe_f32(a, items, classes, s, s1, s2) : launch_chain_mma(a, items, classes, wide, s, s1, s2);
 }
 
 int64_t pipe_image_size(bool f32, int rows, int cols) {

@@ -853,7 +853,7 @@ static void plan_tc(const std::vector<ChainEntry, NoInitAlloc<ChainEntry>> &xs, 
 // Operator images of more than this are given back before a renormalization allocates its block.
 static constexpr size_t kImagesKept = size_t(1) << 30;
 
-// The operators of a position as images (chain_pipe.cu): limbs of the FP64 operators and
+// The operators of a position as images (chain_pipe.cu): digits of the FP64 operators and
 // temporaries, or their FP32 copies.
 struct OpSet {
   DBuf<uint8_t> images;

@@ -63,7 +63,7 @@ struct PsiSpan {
 struct PipeEntry {
   uint64_t x, z;  // byte addresses of the images of X (rows: its rows) and Z (rows: its columns)
   double f;
-  int w;          // limbs: sum of the exponents of X, Z and f (INT_MIN: the task needs FP64)
+  int w;          // digits: sum of the exponents of X, Z and f (INT_MIN: the task needs FP64)
   int src;        // the task in the execution list
 };
 static_assert(sizeof(PipeEntry) == 32, "PipeEntry is 32 bytes");
@@ -74,19 +74,18 @@ struct PipeStack {
   unsigned yb : 24, ns : 4, flags : 4;  // psi block, tasks, whether one of them needs FP64
 };
 static_assert(sizeof(PipeStack) == 16, "the kernel reads a PipeStack as one vector");
-constexpr int kPipeMaxN = 120;  // inner dimension that 64-bit sums of limb products take
+constexpr int kPipeMaxN = 120;  // inner dimension that 64-bit sums of digit products take
 constexpr int kPipeTile = 320;  // elements of the X, Y and Z tiles of the kernel for small blocks
-// Tasks on one psi block that run as one stack: what the tiles of the class's kernel hold (rows of
-// X, depth of T).
+// Tasks on one psi block that run as one stack.  Digits: two, whose X make up the 16 rows of a
+// product.  FP32: what the tiles of the class's kernel hold (rows of X, depth of T).
 #ifdef __CUDACC__
 __host__ __device__
 #endif
-inline int pipe_stack_cap(bool fx, int cls, int m, int q, int n, int p) {
+inline int pipe_stack_cap(bool digits, int cls, int m, int q, int n, int p) {
+  if (digits) return 2;
   if (cls > 1 || n > 32 || p > 32) return 1;
   const bool small = cls == 0;
-  const int pn = fx ? ((n + 1) >> 2 << 2) + 2 : ((n + 3) >> 3 << 3) + 4;
-  const int pp = fx ? ((p + 1) >> 2 << 2) + 2 : ((p + 3) >> 3 << 3) + 4;
-  const int pt = fx ? (p + 1) & ~1 : (p + 3) & ~3;
+  const int pn = ((n + 3) >> 3 << 3) + 4, pp = ((p + 3) >> 3 << 3) + 4, pt = (p + 3) & ~3;
   int c = (small ? 16 : 32) / pt;
   const int rows = 16 / m;
   if (rows < c) c = rows;
@@ -104,8 +103,8 @@ cudaError_t launch_op_images(const OpSlab *s, int nslabs, int64_t nblocks, int16
 cudaError_t launch_psi_images(const PsiSpan *b, int nblocks, const double *psi, void *out, int *exps, bool f32,
                               cudaStream_t st);
 // The tasks of every group (tile0: its kernel class) as PipeEntry and their stacks (from the
-// group's first entry on; nstacks per group); limbs: sorted by psi block within the group.  *bad is set if a task has a form that
-// the kernel does not take.
+// group's first entry on; nstacks per group); digits: sorted by psi block within the group.  *bad is
+// set if a task has a form that the kernels do not take.
 cudaError_t launch_pipe_entries(const ChainEntry *e, const ChainGroup *g, int ngroups, PipeEntry *out,
                                 PipeStack *stacks, int *nstacks, int *bad, const OpTable &ops, const PsiSpan *b,
                                 int nblocks, bool f32, cudaStream_t st);
@@ -116,7 +115,7 @@ struct PipeArgs {
   const ChainEntry *tasks;  // the execution list (FP64 operators: for tasks that fixed point does not take)
   const ChainGroup *g;
   const void *psi;          // images of the psi blocks
-  const int *pexp;          // limbs: their exponents
+  const int *pexp;          // digits: their exponents
   const double *psi64;      // the call's psi
   uint64_t db;
 };
@@ -129,6 +128,9 @@ struct PipeClass {  // the items of a kernel class
 // 1, 3 and 5 on s1, 0 on s2 (the caller orders them; all may be s)
 cudaError_t launch_chain_pipe(const PipeArgs &a, bool f32, const ChainItem *items, const PipeClass *classes, int wide,
                               cudaStream_t s, cudaStream_t s1, cudaStream_t s2);
+// its FP64 part (chain_mma.cu)
+cudaError_t launch_chain_mma(const PipeArgs &a, const ChainItem *items, const PipeClass *classes, int wide,
+                             cudaStream_t s, cudaStream_t s1, cudaStream_t s2);
 
 // Split task lists: every output block's entries are cut into chunks whose
 // partial blocks go to a scratch buffer; this adds them in chunk order.

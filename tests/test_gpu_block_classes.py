@@ -60,7 +60,7 @@ def _close(a, ref, tol):
     return np.max(np.abs(a - ref)) <= tol * np.max(np.abs(ref))
 
 
-SMALL = [(10, c) for c in [(1, 1), (1, 33), (7, 9), (8, 8), (16, 16), (16, 17), (17, 16), (16, 20), (20, 15), (15, 28), (31, 33), (32, 32), (36, 5)]]
+SMALL = [(10, c) for c in [(1, 1), (1, 33), (7, 9), (8, 8), (16, 16), (16, 17), (17, 16), (9, 25), (24, 8), (16, 20), (20, 15), (15, 28), (31, 33), (32, 32), (36, 5)]]
 LARGE = [(12, c) for c in [(33, 64), (65, 63), (96, 97), (100, 100)]]
 
 
