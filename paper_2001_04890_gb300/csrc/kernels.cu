@@ -166,51 +166,46 @@ int dots_partial_blocks(int64_t n) {
   return (int)b;
 }
 
-__global__ void dots_stage1(const double *__restrict__ V, int k, int64_t n,
-                            const double *__restrict__ w, double *partial) {
-  __shared__ double red[32][33];
-  const int nb = gridDim.x;
-  double s[32];
+// Partial dot products of the columns [C blockIdx.y, C blockIdx.y + C) of V with w.  An FP64
+// operation takes a warp 64 clocks of its scheduler, and a vector of 16,600 elements has nine
+// blocks' worth of elements, so the columns go to blocks of their own: 25 columns in one block took
+// 37 us, most of it the reduction over the warp.  That reduction adds lane i + 16 to lane i, then
+// + 8, ... for every column; half of the lanes do one column's additions and half another's as long
+// as there are two, so C columns take C + 1 additions and not 5 C.
+template <int C>
+__global__ void __launch_bounds__(256) dots_stage1(const double *__restrict__ V, int k, int64_t n,
+                                                   const double *__restrict__ w, double *partial) {
+  __shared__ double red[8][C];
+  const int nb = gridDim.x, c0 = C * blockIdx.y, kc = min(C, k - c0);
+  const double *Vc = V + (int64_t)c0 * n;
+  double s[C];
 #pragma unroll
-  for (int j = 0; j < 32; ++j) s[j] = 0.0;
+  for (int j = 0; j < C; ++j) s[j] = 0.0;
+#pragma unroll 2
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)nb * blockDim.x) {
     const double we = w[e];
 #pragma unroll
-    for (int j = 0; j < 32; ++j)
-      if (j < k) s[j] = fma(V[(int64_t)j * n + e], we, s[j]);
+    for (int j = 0; j < C; ++j)
+      if (j < kc) s[j] = fma(Vc[(int64_t)j * n + e], we, s[j]);
   }
-  // Warp sums, every column's by the same tree (lane i + lane i + 16, then + 8, ...).  Up to six
-  // columns each by itself; more of them two at a time per step: half of the lanes add one
-  // column's pairs and half another's, so 31 additions serve 32 columns instead of 160 (an FP64
-  // addition takes a warp 64 clocks here: 37 us of a 16,600-element dot product of 1 to 25
-  // columns was these).
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (k <= 6) {
+  int o = 16;
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      if (j < k) {
-        double x = s[j];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) red[warp][j] = x;
-      }
+  for (int h = C / 2; h > 0; h /= 2, o /= 2) {
+#pragma unroll
+    for (int j = 0; j < h; ++j) {  // columns j (lower lanes) and j + h (upper lanes)
+      const bool up = lane & o;
+      const double give = up ? s[j] : s[j + h], keep = up ? s[j + h] : s[j];
+      s[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
-  } else {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-      for (int j = 0; j < o; ++j) {  // columns j (lower lanes) and j + o (upper lanes)
-        const bool up = lane & o;
-        const double give = up ? s[j] : s[j + o], keep = up ? s[j + o] : s[j];
-        s[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-      }
-    }
-    red[warp][lane] = s[0];  // lane's bits select its column
   }
+  for (; o > 0; o /= 2) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+  if (lane % (32 / C) == 0) red[warp][lane / (32 / C)] = s[0];  // lane's upper bits select its column
   __syncthreads();
-  if (threadIdx.x < k) {
+  if ((int)threadIdx.x < kc) {
     double x = 0.0;
     for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) x += red[w2][threadIdx.x];
-    partial[(int64_t)blockIdx.x * k + threadIdx.x] = x;
+    partial[(int64_t)blockIdx.x * k + c0 + threadIdx.x] = x;
   }
 }
 
@@ -233,7 +228,9 @@ cudaError_t launch_dots(const double *V, int k, int64_t n, const double *w, doub
   if (k <= 0) return cudaSuccess;
   const int nb = dots_partial_blocks(n);
   COUNT(1);
-  dots_stage1<<<nb, 256, 0, s>>>(V, k, n, w, partial);
+  // vectors of few blocks: fewer columns a block; long ones: w is read less often
+  if (nb < 152) dots_stage1<4><<<dim3(nb, (k + 3) / 4), 256, 0, s>>>(V, k, n, w, partial);
+  else dots_stage1<8><<<dim3(nb, (k + 7) / 8), 256, 0, s>>>(V, k, n, w, partial);
   COUNT(1);
   dots_stage2<<<k, 256, 0, s>>>(partial, nb, k, out);
   return cudaGetLastError();
