@@ -353,18 +353,22 @@ cudaError_t launch_fill_guess(double *x, int64_t n, uint64_t seed, cudaStream_t 
 
 // Symmetric eigensolver for the small Davidson subspace matrix (n <= 32):
 // two-sided Jacobi with the round-robin (circle) ordering, so each round
-// applies n/2 disjoint rotations at once (they commute), one thread per pair
-// for the angles and one thread per (row, pair) for the updates.  Rotation
+// applies n/2 disjoint rotations at once (they commute).  Rotation
 // angles as in the classical cyclic method (t = sgn(th)/(|th|+sqrt(th^2+1)),
 // th = (a_qq - a_pp)/(2 a_pq)); sweeps until the off-diagonal norm is below
 // 1e-16 of the diagonal norm.  Eigenvalues ascending; evecs row-major with
 // eigenvector j in column j.
-__global__ void __launch_bounds__(128) jacobi_eigh_kernel(const double *A, int n, int lda, double *evals,
+//
+// One SM's FP64 pipes bound it (an operation takes a warp 64 clocks of its scheduler).  The angles
+// are one warp's chain of divisions and roots, so the other schedulers turn V by the round
+// before meanwhile, and A <- J^T A J is one pass in which a thread has the four elements of two
+// pairs.
+__global__ void __launch_bounds__(256) jacobi_eigh_kernel(const double *A, int n, int lda, double *evals,
                                                           double *evecs) {
   __shared__ double a[32][33];
   __shared__ double v[32][33];
-  __shared__ double rc[16], rs[16];
-  __shared__ int rp[16], rq[16];
+  __shared__ double rc[2][16], rs[2][16];
+  __shared__ int rp[2][16], rq[2][16];  // rq < 0: p has no partner (odd n)
   __shared__ int done;
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int idx = tid; idx < n * n; idx += nt) {
@@ -374,6 +378,19 @@ __global__ void __launch_bounds__(128) jacobi_eigh_kernel(const double *A, int n
   }
   const int N = (n + 1) & ~1;  // an odd n gets a dummy index n (its pairs are skipped)
   const int npair = N / 2;
+  const int warp = tid >> 5, vt = (((warp & 3) - 1) + 3 * (warp >> 2)) * 32 + (tid & 31);  // warps off the first scheduler
+  int cur = 0;
+  bool pending = false;  // V has not seen the rotations of buffer cur ^ 1
+  auto turn_v = [&](int b, int t, int step) {  // V <- V J
+    for (int it = t; it < n * npair; it += step) {
+      const int k = it % n, m = it / n, p = rp[b][m], q = rq[b][m];
+      if (q < 0) continue;
+      const double c = rc[b][m], sn = rs[b][m];
+      const double vkp = v[k][p], vkq = v[k][q];
+      v[k][p] = c * vkp - sn * vkq;
+      v[k][q] = sn * vkp + c * vkq;
+    }
+  };
   __syncthreads();
   for (int sweep = 0; sweep < 60; ++sweep) {
     if (tid < 32) {
@@ -410,37 +427,49 @@ __global__ void __launch_bounds__(128) jacobi_eigh_kernel(const double *A, int n
             sn = t * c;
           }
         } else {
-          p = -1;
+          q = -1;
         }
-        rp[tid] = p;
-        rq[tid] = q;
-        rc[tid] = c;
-        rs[tid] = sn;
+        rp[cur][tid] = p;
+        rq[cur][tid] = q;
+        rc[cur][tid] = c;
+        rs[cur][tid] = sn;
       }
+      if (pending && (warp & 3)) turn_v(cur ^ 1, vt, 192);
       __syncthreads();
-      for (int it = tid; it < n * npair; it += nt) {  // A <- A J, V <- V J
-        const int k = it % n, m = it / n, p = rp[m], q = rq[m];
-        if (p < 0) continue;
-        const double c = rc[m], sn = rs[m];
-        const double akp = a[k][p], akq = a[k][q];
-        a[k][p] = c * akp - sn * akq;
-        a[k][q] = sn * akp + c * akq;
-        const double vkp = v[k][p], vkq = v[k][q];
-        v[k][p] = c * vkp - sn * vkq;
-        v[k][q] = sn * vkp + c * vkq;
+      for (int it = tid; it < npair * npair; it += nt) {  // A <- J^T (A J), rows of pair i, columns of pair j
+        const int i = it / npair, j = it % npair;
+        const int p = rp[cur][i], q = rq[cur][i], y = rp[cur][j], z = rq[cur][j];
+        const double c = rc[cur][i], sn = rs[cur][i], d = rc[cur][j], e = rs[cur][j];
+        double py = a[p][y], pz = 0.0, qy = 0.0, qz = 0.0;
+        if (z >= 0) pz = a[p][z];
+        if (q >= 0) qy = a[q][y];
+        if (q >= 0 && z >= 0) qz = a[q][z];
+        if (z >= 0) {
+          const double u = py, w = qy;
+          py = d * u - e * pz;
+          pz = e * u + d * pz;
+          qy = d * w - e * qz;
+          qz = e * w + d * qz;
+        }
+        if (q >= 0) {
+          const double u = py, w = pz;
+          py = c * u - sn * qy;
+          qy = sn * u + c * qy;
+          pz = c * w - sn * qz;
+          qz = sn * w + c * qz;
+        }
+        a[p][y] = py;
+        if (z >= 0) a[p][z] = pz;
+        if (q >= 0) a[q][y] = qy;
+        if (q >= 0 && z >= 0) a[q][z] = qz;
       }
-      __syncthreads();
-      for (int it = tid; it < n * npair; it += nt) {  // A <- J^T A
-        const int k = it % n, m = it / n, p = rp[m], q = rq[m];
-        if (p < 0) continue;
-        const double c = rc[m], sn = rs[m];
-        const double apk = a[p][k], aqk = a[q][k];
-        a[p][k] = c * apk - sn * aqk;
-        a[q][k] = sn * apk + c * aqk;
-      }
+      cur ^= 1;
+      pending = true;
       __syncthreads();
     }
   }
+  if (pending) turn_v(cur ^ 1, tid, nt);
+  __syncthreads();
   if (tid == 0) {
     for (int i = 0; i < n; ++i) {
       int m = i;
@@ -467,7 +496,7 @@ cudaError_t launch_jacobi_eigh(const double *A, int n, int lda, double *evals, d
                                cudaStream_t s) {
   if (n > 32 || n < 1) return cudaErrorInvalidValue;
   COUNT(1);
-  jacobi_eigh_kernel<<<1, 128, 0, s>>>(A, n, lda, evals, evecs);
+  jacobi_eigh_kernel<<<1, 256, 0, s>>>(A, n, lda, evals, evecs);
   return cudaGetLastError();
 }
 
