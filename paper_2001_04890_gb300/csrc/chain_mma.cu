@@ -25,10 +25,17 @@
 // registers, so a lane's share of an 8 x 16 block is three 128-bit loads and digits need no shared
 // memory, no transposition and no barrier; lines are asked for one task ahead.  T comes out of the
 // first product in the layout that the second one takes as its B operand, so for up to 32
-// columns it never leaves the registers: D^T = sum Z^T T^T.
+// columns it never leaves the registers: D^T = sum Z^T T^T.  It is made 16 columns at a time:
+// the sums of 32 want registers that the second product needs (24 orbitals, M 512: 8.7 against
+// 8.2 ms, 12, M 800: 18.0 against 15.9 ms at equal occupancy), though D is then added to twice as
+// often.
 //
-// Time per H psi, limbs on the integer pipe -> this: 8 orbitals, M 64: 196 -> 181 us; 11, M 150:
-// 585 -> 396 us; 24, M 512: 11.2 -> 8.7 ms; 12, M 800: 23.1 -> 18.5 ms.
+// What bounds it: latency.  229 instructions a multiply of 26 (sums to integers, digits of T, D)
+// keep the tensor pipe 28% busy at 3 warps a scheduler, and registers allow 4.  Blocks are padded
+// to 16 x 8 x 8: a third of the products at 24 orbitals, M 512, are of the problem.
+//
+// Time per H psi, limbs on the integer pipe -> this: 8 orbitals, M 64: 196 -> 179 us; 11, M 150:
+// 585 -> 357 us; 24, M 512: 11.2 -> 7.6 ms; 12, M 800: 23.1 -> 15.2 ms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -98,10 +105,10 @@ __device__ __forceinline__ void load_rows(const char *p, bool full, const char *
 }
 
 // 1.5 2^23: the low bits of its sum with an integer below 2^22 are that integer.  G_0 and G_1 start
-// from it, which saves them a conversion; the sums begin with what it adds up to taken off.
+// from it, which saves them a conversion; the sum begins with what it adds taken off.
 constexpr float kMagic = 12582912.f;
 constexpr unsigned long long kMagicBits = 0x4b400000ull;
-constexpr unsigned long long kMagicSum = (kMagicBits << 40) + (kMagicBits << 30);  // of one depth of 16
+constexpr unsigned long long kMagicSum = (kMagicBits << 40) + (kMagicBits << 30);  
 
 // Powers of two as values the compiler does not know: a multiply-add is one instruction, the shift
 // and the 64-bit addition that it would make of it are four.
@@ -126,7 +133,7 @@ __device__ __forceinline__ void sums(const uint32_t (&a)[6][4], const uint32_t (
     }
 }
 
-// s += a b (16 rows, 8 columns) over a depth of 16, or 8 (half)
+// s = a b (16 rows, 8 columns) over a depth of 16, or 8 (half)
 __device__ __forceinline__ void multiply(const uint32_t (&a)[6][4], const uint32_t (&b)[6][2], bool half, const Powers &w,
                                          long long (&s)[4]) {
   float g[7][4];
@@ -134,6 +141,7 @@ __device__ __forceinline__ void multiply(const uint32_t (&a)[6][4], const uint32
   else sums<false>(a, b, g);
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
+    s[e] = (long long)(0ull - kMagicSum);
     // units of 2^60: G_0 2^40 + G_1 2^30 + G_2 2^20 + G_3 2^10 + (G_4 + G_5 2^-10 + G_6 2^-20)
     mad(s[e], __float2int_rn(fmaf(fmaf(g[6][e], 0x1p-10f, g[5][e]), 0x1p-10f, g[4][e])), w.p0);
     mad(s[e], __float2int_rn(g[3][e]), w.p10);
@@ -144,19 +152,17 @@ __device__ __forceinline__ void multiply(const uint32_t (&a)[6][4], const uint32
   }
 }
 
-// Digits of T, rows of one 8-row block: t[j][0..1] = columns 8 j + 2 (lane & 3) and the next one;
-// out[ks] = the block of columns 16 ks.. (those below depth), as load_block gives it.  Returns
-// the shift that took T to 58 bits.
-template <int OFF, int NJ>
-__device__ __forceinline__ int digits_of(const long long (&t)[NJ][4], int depth, uint32_t (&out)[NJ / 2][6][2]) {
+// Digits of 8 rows and 16 columns of T: t[j][OFF + i] = column 8 j + 2 (lane & 3) + i of row lane / 4;
+// out = the block as load_block gives it.  Returns the shift that took T to 58 bits.
+template <int OFF>
+__device__ __forceinline__ int digits_of(const long long (&t)[2][4], uint32_t (&out)[6][2]) {
   unsigned mx = 0;
 #pragma unroll
-  for (int j = 0; j < NJ; ++j) mx = max(mx, max(magnitude(t[j][OFF]), magnitude(t[j][OFF + 1])));
+  for (int j = 0; j < 2; ++j) mx = max(mx, max(magnitude(t[j][OFF]), magnitude(t[j][OFF + 1])));
   mx = __reduce_max_sync(kFull, mx);
   const int up = __clz(mx | 1) - 6;
 #pragma unroll
-  for (int j = 0; j < NJ; ++j) {
-    if (j % 2 == 0 && 8 * j >= depth) break;
+  for (int j = 0; j < 2; ++j) {
     long long v = t[j][OFF], w = t[j][OFF + 1];
     if (up >= 0) {
       v <<= up;
@@ -169,7 +175,7 @@ __device__ __forceinline__ int digits_of(const long long (&t)[NJ][4], int depth,
     uint32_t d[6];
     digits2(v, w, d);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) out[j >> 1][i][j & 1] = d[i];
+    for (int i = 0; i < 6; ++i) out[i][j] = d[i];
   }
   return up;
 }
@@ -218,22 +224,16 @@ __device__ __noinline__ void slow_stacks(const PipeEntry *P, const PipeStack *S,
   }
 }
 
-// Warps an SM holds: registers against latency.  Blocks of at most 16 columns at 12 / 16 / 20 warps: H
-// psi, 8 orbitals, M 64: 181 / 196 / 217 us; Davidson, 10 orbitals, M 128: 115 / 132 / 131 ms;
-// 16 vectors, 24 orbitals, M 512: 12.8 / 11.7 / 11.9 ms.  Wider ones at 12 / 16: 24 orbitals, M
-// 512: 8.6 / 8.4 ms; 12 orbitals, M 800: 18.5 / 22.5 ms.
-constexpr int kSmWarps = 12;
-
 // One 16-row slice of a work item per CTA: rows [r0, r0 + 16) (slice blockIdx.y) and columns
 // [c0, c0 + 16 NQ WC) of one chunk's output block.  A warp has 16 NQ columns.  WC = 1: the
 // warps of the CTA take the chunk's stacks in turn, each by itself; their sums are added in
-// warp order.  WC > 1: the WC warps each compute 8 NJ columns of T, share the digits through
+// warp order.  WC > 1: the WC warps each compute 16 columns of T, share the digits through
 // shared memory and multiply them with their own columns of Z.
 //
 // A task at a time, or, for a slice of at most 8 rows, two tasks of a stack at a time: they
 // share Y, so their X make up the 16 rows of the first product.
-template <int NQ, int NJ, int WC>
-__global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ? 4 : WC))
+template <int NQ, int WC, int SMW>
+__global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, SMW / (WC == 1 ? 4 : WC))
     chain_mma_kernel(const PipeEntry *__restrict__ E, const PipeStack *__restrict__ stacks,
                      const int *__restrict__ nstacks, const ChainEntry *__restrict__ tasks,
                      const ChainGroup *__restrict__ G, const ChainItem *__restrict__ items,
@@ -241,7 +241,6 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ?
                      uint64_t db, Powers w) {
   extern __shared__ __align__(16) unsigned char mma_smem[];
   __shared__ int te[2][WC][2];  // WC > 1: shifts of the chunks of T
-  constexpr int NK = NJ / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wcol = WC == 1 ? 0 : warp;
   const int grp = WC == 1 ? warp : 0, ngrp = WC == 1 ? (int)(blockDim.x >> 5) : 1;
@@ -265,24 +264,33 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ?
   bool any_special = false;
   int buf = 0;  // WC > 1: buffer of T
 
-  // a stack as read, and the exponent of its Y
-  int4 d = make_int4(0, 0, 0, 0);
+  // The stack at hand and the exponent of its Y, and the next one as read: when its turn comes it is
+  // here, and what it points to is asked for while the tasks before it are computed.
+  int4 d, nd;
   int si = grp, mem = 0, ey = 0, ns = 0;
-  auto take = [&]() {  // the next stack that fixed point takes; ns = 0: none
-    for (;;) {
-      ns = 0;
-      if (si >= nst) return;
-      d = *reinterpret_cast<const int4 *>(stk + si);
-      si += ngrp;
-      ey = pexp[d.w & 0xffffff];
-      ns = (d.w >> 24) & 15;
-      if (ey >= 0 && (unsigned)d.w >> 28 == 0) return;
-      any_special = true;
-    }
+  auto read = [&]() {
+    nd = si < nst ? *reinterpret_cast<const int4 *>(stk + si) : make_int4(0, 0, 0, 0);
+    si += ngrp;
   };
-  take();
+  auto next = [&]() {  // ns = 0: no further stack
+    d = nd;
+    ns = (d.w >> 24) & 15;
+    mem = 0;
+    if (ns > 0) {
+      ey = pexp[d.w & 0xffffff];
+      prefetch(E + d.x);
+    }
+    read();
+  };
+  read();
+  next();
 #pragma unroll 1
   while (ns > 0) {
+    if (mem == 0 && (ey < 0 || (unsigned)d.w >> 28 != 0)) {  // not in fixed point
+      any_special = true;
+      next();
+      continue;
+    }
     const int n = d.y & 0xffff, p = (int)((unsigned)d.y >> 16), rby = (p + 7) >> 3;
     const char *Y = psi + (uint64_t)(uint32_t)d.z * 8;
     const PipeEntry *e0 = E + d.x + mem;
@@ -292,13 +300,8 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ?
     const char *Z0 = reinterpret_cast<const char *>(e0->z) + (c0 >> 3) * kDigBlock;
     const char *Z1 = two ? reinterpret_cast<const char *>(e0[1].z) + (c0 >> 3) * kDigBlock : Z0;
     const int ney = ey;
-    // what the task after this one reads
     mem += pair ? 2 : 1;
-    if (mem >= ns) {
-      mem = 0;
-      take();
-    }
-    if (ns > 0) prefetch(E + d.x + mem);
+    if (mem >= ns) next();  // from here on d, mem, ey and ns are those of the next task
     for (int k = 0; k < p; k += 16) {
       const int o = (k >> 4) * rbz * kDigBlock, lines = min(2 * NQ, rbz - (c0 >> 3)) * (kDigBlock / 128);
       for (int i = lane; i < lines; i += 32) {
@@ -307,17 +310,13 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ?
       }
     }
 #pragma unroll 1
-    for (int pb = 0; pb < p; pb += 8 * NJ * WC) {
-      uint32_t td[2][NK][6][2];  // digits of T: [8 rows][16 columns]
+    for (int pb = 0; pb < p; pb += 16 * WC) {
+      uint32_t td[2][6][2];  // digits of T: [8 rows]
       int up0 = 0, up1 = 0;
-      const int pm = pb + 8 * NJ * wcol;  // this warp's columns of T
+      const int pm = pb + 16 * wcol;  // this warp's columns of T
       if (pm < p) {
-        long long t[NJ][4];
-#pragma unroll
-        for (int j = 0; j < NJ; ++j)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) t[j][e] = 0;
-        const int nj = min(NJ, rby - (pm >> 3));
+        long long t[2][4] = {};
+        const int nj = min(2, rby - (pm >> 3));
 #pragma unroll 1
         for (int k = 0; k < n; k += 16) {
           uint32_t a[6][4];
@@ -329,19 +328,17 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ?
             uint32_t b[6][2];
             load_block(Yk + j * kDigBlock, lane, b);
             long long s[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) s[e] = (long long)(0ull - kMagicSum);
             multiply(a, b, half, w, s);
 #pragma unroll
-            for (int u = 0; u < NJ; ++u)
+            for (int u = 0; u < 2; ++u)
               if (u == j) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) t[u][e] += s[e];
               }
           }
         }
-        up0 = digits_of<0>(t, p - pm, td[0]);
-        if (x1) up1 = digits_of<2>(t, p - pm, td[1]);
+        up0 = digits_of<0>(t, td[0]);
+        if (x1) up1 = digits_of<2>(t, td[1]);
       }
       if (pb == 0 && ns > 0) {  // X and Y of the next task
         const int nn = d.y & 0xffff, np = (int)((unsigned)d.y >> 16);
@@ -359,18 +356,15 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ?
           for (int i = lane; i < lines; i += 32) prefetch(y + i * 128);
         }
       }
-      const int nc = WC == 1 ? 1 : min(WC, (p - pb + 8 * NJ - 1) / (8 * NJ));
+      const int nc = WC == 1 ? 1 : min(WC, (p - pb + 15) / 16);
       if constexpr (WC > 1) {
-        uint4 *Ts = reinterpret_cast<uint4 *>(mma_smem + (buf * WC + wcol) * (2 * NK * kDigBlock));
+        uint4 *Ts = reinterpret_cast<uint4 *>(mma_smem + (buf * WC + wcol) * (2 * kDigBlock));
         if (pm < p) {
 #pragma unroll
           for (int b = 0; b < 2; ++b)
 #pragma unroll
-            for (int ks = 0; ks < NK; ++ks)
-#pragma unroll
-              for (int v = 0; v < 3; ++v)
-                Ts[((b * NK + ks) * 3 + v) * 32 + lane] =
-                    make_uint4(td[b][ks][2 * v][0], td[b][ks][2 * v][1], td[b][ks][2 * v + 1][0], td[b][ks][2 * v + 1][1]);
+            for (int v = 0; v < 3; ++v)
+              Ts[(b * 3 + v) * 32 + lane] = make_uint4(td[b][2 * v][0], td[b][2 * v][1], td[b][2 * v + 1][0], td[b][2 * v + 1][1]);
           if (lane == 0) {
             te[buf][wcol][0] = up0;
             te[buf][wcol][1] = up1;
@@ -380,42 +374,31 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, kSmWarps / (WC == 1 ?
       }
 #pragma unroll 1
       for (int c = 0; c < nc; ++c) {
-        const int pc0 = pb + 8 * NJ * c;
+        const int pc = pb + 16 * c;
         if constexpr (WC > 1) {
-          const char *Ts = reinterpret_cast<const char *>(mma_smem + (buf * WC + c) * (2 * NK * kDigBlock));
+          const char *Ts = reinterpret_cast<const char *>(mma_smem + (buf * WC + c) * (2 * kDigBlock));
 #pragma unroll
-          for (int b = 0; b < 2; ++b)
-#pragma unroll
-            for (int ks = 0; ks < NK; ++ks) load_block(Ts + (b * NK + ks) * kDigBlock, lane, td[b][ks]);
+          for (int b = 0; b < 2; ++b) load_block(Ts + b * kDigBlock, lane, td[b]);
           up0 = te[buf][c][0];
           up1 = te[buf][c][1];
         }
-        const int depth = min(8 * NJ, p - pc0);
         // 2^60 T64 = 2^(60 - up) T, and the same units again; f's exponent is in the entry's w
         const double f0 = e0->f, f1 = two ? e0[1].f : f0;
         const int s0 = 120 - 3240 - 1023 + ney - up0 + e0->w, s1 = 120 - 3240 - 1023 + ney - up1 + (two ? e0[1].w : e0->w);
         const double q0 = __hiloint2double((__double2hiint(f0) & 0x800fffff) | ((s0 + 1023) << 20), __double2loint(f0));
         const double q1 = __hiloint2double((__double2hiint(f1) & 0x800fffff) | ((s1 + 1023) << 20), __double2loint(f1));
+        const bool half = p - pc <= 8;
 #pragma unroll 1
         for (int j = 0; 16 * j < q; ++j) {
-          long long s[2][4];
-          const long long start = (long long)(0ull - kMagicSum * (unsigned)((depth + 15) >> 4));
-#pragma unroll
-          for (int e = 0; e < 4; ++e) s[0][e] = s[1][e] = start;
           const bool have = (c0 >> 3) + 2 * j + 1 < rbz;
-#pragma unroll
-          for (int ks = 0; ks < NK; ++ks) {
-            if (16 * ks < depth) {
-              const bool half = depth - 16 * ks <= 8;
-              const int off = (((pc0 >> 4) + ks) * rbz + 2 * j) * kDigBlock;
-              uint32_t a[6][4];
-              load_rows(Z0 + off, have, Z0, false, lane, a);
-              multiply(a, td[0][ks], half, w, s[0]);
-              if (x1) {
-                if (two) load_rows(Z1 + off, have, Z1, false, lane, a);
-                multiply(a, td[1][ks], half, w, s[1]);
-              }
-            }
+          const int off = ((pc >> 4) * rbz + 2 * j) * kDigBlock;
+          uint32_t a[6][4];
+          load_rows(Z0 + off, have, Z0, false, lane, a);
+          long long s[2][4];
+          multiply(a, td[0], half, w, s[0]);
+          if (x1) {
+            if (two) load_rows(Z1 + off, have, Z1, false, lane, a);
+            multiply(a, td[1], half, w, s[1]);
           }
 #pragma unroll
           for (int u = 0; u < NQ; ++u)
@@ -478,16 +461,18 @@ int warps_per_slice(int n, int64_t tasks, int resident) {
   return k;
 }
 
-template <int NQ, int NJ, int WC>
+// SMW: warps that an SM holds, registers against latency.  At 12 a warp has the 168 registers
+// that its sums, fragments and addresses want; at 16 it spills some outside the products, which
+// pays where there are warps enough.  12 / 16 for more than 32 columns: 12 orbitals, M 800: 16.3 /
+// 15.2 ms; for 32: 24 orbitals, M 512: 8.2 / 7.7 ms.
+template <int NQ, int WC, int SMW>
 cudaError_t launch_mma(const PipeArgs &a, const ChainItem *items, const PipeClass &c, int slices, bool share,
                        cudaStream_t s) {
   if (c.items <= 0) return cudaSuccess;
-  const int warps = WC > 1 ? WC : share ? warps_per_slice(c.items * slices, c.tasks, kSmWarps * 152) : 1;
+  const int warps = WC > 1 ? WC : share ? warps_per_slice(c.items * slices, c.tasks, SMW * 152) : 1;
   // T of WC > 1 (two buffers), the sums of a warp, or T of slow_stacks
-  const int bytes = std::max({WC > 1 ? 2 * WC * NJ * kDigBlock : 0, 8 * NQ * 32 * 8, 16 * 16 * 8});
-  auto kern = chain_mma_kernel<NQ, NJ, WC>;
-  const cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (err != cudaSuccess) return err;
+  const int bytes = std::max({WC > 1 ? 2 * WC * 2 * kDigBlock : 0, 8 * NQ * 32 * 8, 16 * 16 * 8});
+  auto kern = chain_mma_kernel<NQ, WC, SMW>;
   add_kernel_launches(1);
   kern<<<dim3(c.items, slices), 32 * warps, bytes, s>>>(a.e, a.stacks, a.nstacks, a.tasks, a.g, items,
                                                         static_cast<const char *>(a.psi), a.pexp, a.psi64, a.db,
@@ -506,12 +491,15 @@ cudaError_t launch_chain_mma(const PipeArgs &a, const ChainItem *items, const Pi
     return p;
   };
   const ChainItem *i5 = next(5), *i4 = next(4), *i3 = next(3), *i2 = next(2), *i1 = next(1), *i0 = next(0);
-  if ((err = launch_mma<2, 4, 4>(a, i5, c[5], 2, false, s1)) != cudaSuccess) return err;
-  if ((err = launch_mma<2, 4, 3>(a, i4, c[4], 2, false, s)) != cudaSuccess) return err;
-  if ((err = launch_mma<2, 4, 2>(a, i3, c[3], 2, false, s1)) != cudaSuccess) return err;
-  if ((err = launch_mma<2, 4, 1>(a, i2, c[2], 2, wide != 0, s)) != cudaSuccess) return err;
-  if ((err = launch_mma<2, 4, 1>(a, i1, c[1], 1, wide != 0, s1)) != cudaSuccess) return err;
-  return launch_mma<1, 2, 1>(a, i0, c[0], 1, wide != 0, s2);
+  if ((err = launch_mma<2, 4, 16>(a, i5, c[5], 2, false, s1)) != cudaSuccess) return err;
+  if ((err = launch_mma<2, 3, 15>(a, i4, c[4], 2, false, s)) != cudaSuccess) return err;
+  if ((err = launch_mma<2, 2, 16>(a, i3, c[3], 2, false, s1)) != cudaSuccess) return err;
+  if ((err = launch_mma<2, 1, 16>(a, i2, c[2], 2, wide != 0, s)) != cudaSuccess) return err;
+  if ((err = launch_mma<2, 1, 16>(a, i1, c[1], 1, wide != 0, s1)) != cudaSuccess) return err;
+  // 12 / 16: 8 orbitals, M 64 (459 items): 181 / 196 us; 16 vectors, 24 orbitals, M 512 (14,368):
+  // 12.2 / 11.2 ms.  An item has four warps at most: the line is two waves of 16 an SM.
+  if (c[0].items > 2 * 4 * 152) return launch_mma<1, 1, 16>(a, i0, c[0], 1, wide != 0, s2);
+  return launch_mma<1, 1, 12>(a, i0, c[0], 1, wide != 0, s2);
 }
 
 }  // namespace dmrg
