@@ -61,16 +61,12 @@ for _key, _wl in WORKLOADS.items():
 
 DAVIDSON_ITERS_PER_STEP = 4  # working-precision Davidson iterations per timed step
 
-FP64_NOMINAL_TFLOPS = 1.25  # GB300 FP64 (nominal, recipe table)
+FP64_PASSES = 26  # FP16 tensor-core products per product of 58-bit integers (chain_mma.cu)
 FP32_SIMT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12  # FP32 FMA units x 2 FLOP x max SM clock
 
 # DRAM bytes (read + write) per launch of the dominant H.psi kernel, from one ncu
 # capture of the unchanged kernel at that workload and precision (else null)
 TRAFFIC_PER_LAUNCH = {
-    ("c2", 0, 512, (32768.0, 50000.0, 33, 0, 0, 0)): 1.034e9 + 0.147e9,
-    ("c2", 0, 512, (32768.0, 200000.0, 33, 0, 0, 0)): 1.0293e9 + 0.1472e9,
-    ("c2", 0, 512, (131072.0, 50000.0, 33, 0, 0, 0)): 1.8010e9 + 0.7325e9,
-    ("c2", 0, 512, (131072.0, 200000.0, 33, 0, 0, 0)): 1.4767e9 + 0.4892e9,
     # split-BF16x3 H.psi, every block on the tensor cores: DRAM read + write of the
     # chain_tc2 launches of one H.psi (one shape at M=3000, two at M=6000)
     ("c5a", 2, 3000, (8192.0, 200000.0, 1, 1, 1, 0)): 434.8e9 + 0.175e9,
@@ -143,6 +139,13 @@ def _peaks():
         return json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
     except OSError:
         return {}
+
+
+def _fp64_peak(peaks):
+    peak = peaks.get("bf16_tflops")
+    return {"bound": "tensor", "peak": peak / FP64_PASSES if peak else None, "unit": "TFLOP/s",
+            "peak_source": f"MEASURED_PEAKS.json bf16_tflops (burst) / {FP64_PASSES}: FP16 products of digits per"
+                           " FP64 product (of measured; mma.sync reaches a quarter of that rate)"}
 
 
 def _oracle_workload(wl):
@@ -817,9 +820,11 @@ def davidson_line(args, wl, rank, world, prec):
                 "peak_source": "MEASURED_PEAKS.json bf16_tflops (burst) / 3: three bf16 passes per product"
                                " (of measured)",
                 "unit": "TFLOP/s"}
+    elif prec == 0:
+        roof = {"kernel": "chain_mma_kernel (H.psi)", "achieved": kernel_tflops, **_fp64_peak(peaks)}
     else:
-        roof = {"bound": "alu", "kernel": "chain kernels (SIMT)", "achieved": kernel_tflops,
-                "peak": FP64_NOMINAL_TFLOPS if prec == 0 else FP32_SIMT_TFLOPS,
+        roof = {"bound": "alu", "kernel": "chain_pipe_kernel (H.psi, FP32 operators)", "achieved": kernel_tflops,
+                "peak": FP32_SIMT_TFLOPS,
                 "peak_source": "unit counts x 2.07 GHz (no measured SIMT peak)", "unit": "TFLOP/s"}
     roof["frac"] = (kernel_tflops / roof["peak"]) if (kernel_tflops and roof["peak"]) else None
     roof["traffic"] = TRAFFIC_PER_LAUNCH.get((args.workload, prec, wl["M"], _shape_key(r["tune"])))
@@ -884,6 +889,7 @@ def fp64_step_line(args, wl, rank, world):
     value = whole_job_tflops(hpsi_flops, world, r["step_ms"])
     kernel_tflops = st["hpsi_flops"] / (st["hpsi_ms"] * 1e-3) / 1e12 if st["hpsi_ms"] > 0 else None
     dav_iters = st["davidson_iters"]
+    fp64_peak = _fp64_peak(_peaks())
     line = {
         "metric": METRIC,
         "value": value,
@@ -909,13 +915,10 @@ def fp64_step_line(args, wl, rank, world):
         "hpsi_plan_s": r["plan_s"],
         "energy": r["energy"],
         "roofline": {
-            "bound": "alu",
-            "kernel": "chain_flat_kernel<double> (H.psi)",
+            "kernel": "chain_mma_kernel (H.psi)",
             "achieved": kernel_tflops,
-            "peak": FP64_NOMINAL_TFLOPS,
-            "peak_source": "nominal GB300 FP64 from the recipe table (no measured FP64 peak in MEASURED_PEAKS.json)",
-            "unit": "TFLOP/s",
-            "frac": (kernel_tflops / FP64_NOMINAL_TFLOPS) if kernel_tflops else None,
+            **fp64_peak,
+            "frac": (kernel_tflops / fp64_peak["peak"]) if kernel_tflops and fp64_peak["peak"] else None,
             "traffic": TRAFFIC_PER_LAUNCH.get((wl.get("key", ""), 0, wl["M"], _shape_key(r["tune"]))),
         },
         "e2e": {"value": hpsi_flops / (r["e2e_ms"] * 1e-3) / 1e12, "unit": "TFLOP/s",

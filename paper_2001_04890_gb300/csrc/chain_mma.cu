@@ -30,8 +30,8 @@
 // 8.2 ms, 12, M 800: 18.0 against 15.9 ms at equal occupancy), though D is then added to twice as
 // often.
 //
-// What bounds it: latency.  229 instructions a multiply of 26 (sums to integers, digits of T, D)
-// keep the tensor pipe 28% busy at 3 warps a scheduler, and registers allow 4.  Blocks are padded
+// What bounds it: latency.  225 instructions a multiply of 26 (sums to integers, digits of T, D)
+// keep the tensor pipe 24 to 32% busy at the 4 warps a scheduler that registers allow.  Blocks are padded
 // to 16 x 8 x 8: a third of the products at 24 orbitals, M 512, are of the problem.
 //
 // Time per H psi, limbs on the integer pipe -> this: 8 orbitals, M 64: 196 -> 179 us; 11, M 150:
