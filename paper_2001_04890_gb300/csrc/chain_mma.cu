@@ -303,7 +303,8 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, SMW / (WC == 1 ? 4 : 
     mem += pair ? 2 : 1;
     if (mem >= ns) next();  // from here on d, mem, ey and ns are those of the next task
     for (int k = 0; k < p; k += 16) {
-      const int o = (k >> 4) * rbz * kDigBlock, lines = min(2 * NQ, rbz - (c0 >> 3)) * (kDigBlock / 128);
+      const int64_t o = (int64_t)(k >> 4) * rbz * kDigBlock;
+      const int lines = min(2 * NQ, rbz - (c0 >> 3)) * (kDigBlock / 128);
       for (int i = lane; i < lines; i += 32) {
         prefetch(Z0 + o + i * 128);
         if (two) prefetch(Z1 + o + i * 128);
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, SMW / (WC == 1 ? 4 : 
 #pragma unroll 1
         for (int j = 0; 16 * j < q; ++j) {
           const bool have = (c0 >> 3) + 2 * j + 1 < rbz;
-          const int off = ((pc >> 4) * rbz + 2 * j) * kDigBlock;
+          const int64_t off = (int64_t)((pc >> 4) * rbz + 2 * j) * kDigBlock;
           uint32_t a[6][4];
           load_rows(Z0 + off, have, Z0, false, lane, a);
           long long s[2][4];
