@@ -498,7 +498,7 @@ cudaError_t launch_chain_mma(const PipeArgs &a, const ChainItem *items, const Pi
   if ((err = launch_mma<2, 1, 16>(a, i2, c[2], 2, wide != 0, s)) != cudaSuccess) return err;
   if ((err = launch_mma<2, 1, 16>(a, i1, c[1], 1, wide != 0, s1)) != cudaSuccess) return err;
   // 12 / 16: 8 orbitals, M 64 (459 items): 181 / 196 us; 16 vectors, 24 orbitals, M 512 (14,368):
-  // 12.2 / 11.2 ms.  An item has four warps at most: the line is two waves of 16 an SM.
+  // 11.9 / 10.8 ms.  An item has four warps at most: the line is two waves of 16 an SM.
   if (c[0].items > 2 * 4 * 152) return launch_mma<1, 1, 16>(a, i0, c[0], 1, wide != 0, s2);
   return launch_mma<1, 1, 12>(a, i0, c[0], 1, wide != 0, s2);
 }
