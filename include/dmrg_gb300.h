@@ -506,6 +506,19 @@ int dmrg_plan_hpsi_flops(int L, int N, int two_sz, const double *h, const double
 int dmrg_selftest_tcgen05(int N, int K, const float *A, const float *B, float *C);
 
 /*
+ * dmrg_selftest_chain -- device check of the triple products that the task lists
+ * consist of (diagnostic; Eq. dgemm): D (m x q) = sum_t f[t] X_t Y Z_t, X ntasks
+ * x m x n, Y n x p, Z ntasks x p x q.  X or Z may be NULL: the identity (n = m,
+ * p = q).  kind: 0 FP64 as H.psi runs it on prepared operands, 1 FP64 as the
+ * other products and H.psi without room for those run, 2 and 3 the same with
+ * FP32 operators.  Host pointers, row-major.  DMRG_EINVAL for sides outside
+ * 1..1024, more than 4096 tasks or 2^24 operator elements, or (kinds 0, 2) an
+ * inner dimension that the prepared kernels do not take.
+ */
+int dmrg_selftest_chain(int kind, int ntasks, int m, int n, int p, int q, const double *X, const double *Y,
+                        const double *Z, const double *f, double *D);
+
+/*
  * dmrg_debug_set_wait_limit -- fault detection test hook (no paper
  * counterpart), process-wide.  Sets the number of polls of every pipeline wait
  * of the tensor-core kernel (a job's operands landed, a stage freed, T or D

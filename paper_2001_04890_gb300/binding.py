@@ -69,6 +69,7 @@ def lib():
                                            C.c_int, ip, dp, llp]),
         "dmrg_selftest_tcgen05": (C.c_int, [C.c_int, C.c_int, C.POINTER(C.c_float), C.POINTER(C.c_float),
                                             C.POINTER(C.c_float)]),
+        "dmrg_selftest_chain": (C.c_int, [C.c_int] * 6 + [dp] * 5),
         "dmrg_batch_create": (C.c_int, [C.c_int, C.POINTER(vp), C.POINTER(vp)]),
         "dmrg_batch_layout": (C.c_int, [vp, llp, dp]),
         "dmrg_batch_hpsi": (C.c_int, [vp, vp, vp, C.c_int]),
@@ -289,6 +290,24 @@ def selftest_tcgen05(A, B):
     fp = C.POINTER(C.c_float)
     _check(lib().dmrg_selftest_tcgen05(N, K, A.ctypes.data_as(fp), B.ctypes.data_as(fp), Cm.ctypes.data_as(fp)))
     return Cm
+
+
+def selftest_chain(X, Y, Z, f, fp32=False, prepared=True):
+    """sum_t f_t X_t Y Z_t through the kernels of the task lists.  X: tasks x m x n or None (identity),
+    Y: n x p, Z: tasks x p x q or None.  prepared: the H.psi kernels on operand images, else the
+    general ones; fp32: FP32 operators."""
+    f, Y = _f64(f), _f64(Y)
+    n, p = Y.shape
+    X, Z = (None if a is None else _f64(a) for a in (X, Z))
+    m = n if X is None else X.shape[1]
+    q = p if Z is None else Z.shape[2]
+    if (X is not None and X.shape != (len(f), m, n)) or (Z is not None and Z.shape != (len(f), p, q)):
+        raise ValueError("X is tasks x m x n, Z is tasks x p x q")
+    D = np.zeros((m, q))
+    _check(lib().dmrg_selftest_chain(2 * bool(fp32) + (not prepared), len(f), m, n, p, q,
+                                     None if X is None else _dptr(X), _dptr(Y), None if Z is None else _dptr(Z),
+                                     _dptr(f), _dptr(D)))
+    return D
 
 
 def debug_pieces(h, v, k, l_empty, r_empty, compress=True):

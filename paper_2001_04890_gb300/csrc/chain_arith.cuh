@@ -85,11 +85,15 @@ struct TileMax {
     any |= h | (unsigned)__double2loint(x);
   }
 };
-// exponents that fixed point takes; an all-zero tile counts as exponent 0
-__device__ __forceinline__ bool tile_special(unsigned hi, unsigned any) {
-  const unsigned E = hi >> 20;
-  return E > 1023u + 256u || (E < 1023u - 256u && any != 0u);
+// The exponent of a tile: that of its largest element, -1 if fixed point does not take it, 0 if
+// every element is zero.  Scale factors are made of exponents by integer additions to the exponent
+// field and stay normal numbers for any that lie within 2^+-256; zero_as_one() gives them one for
+// a tile of zeros, whose integers are zero under any exponent.
+__device__ __forceinline__ int tile_exponent(unsigned hi, unsigned any) {
+  const int E = (int)(hi >> 20);
+  return any == 0u ? 0 : E > 1023 + 256 || E < 1023 - 256 ? -1 : E;
 }
+__device__ __forceinline__ int zero_as_one(int E) { return E == 0 ? 1023 : E; }
 
 template <int TS>
 struct Shift {
@@ -212,7 +216,7 @@ __device__ __forceinline__ void mm_any(const float *A, int pa, const float *B, i
 
 __device__ __forceinline__ unsigned magnitude(long long t) { return (unsigned)((t ^ (t >> 63)) >> 32); }
 
-// f 2^e for an f whose exponent is moderate (|e| stays below 1000, see tile_special)
+// f 2^e for an f whose exponent is moderate (|e| stays below 1000, see tile_exponent)
 __device__ __forceinline__ double scaled(double f, int e) {
   return __hiloint2double(__double2hiint(f) + (e << 20), __double2loint(f));
 }

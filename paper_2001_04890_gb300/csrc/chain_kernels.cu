@@ -108,15 +108,14 @@ __device__ __forceinline__ void raw_to_limbs(int2 *tile, const View<TS> &V, int 
   pad_tile<true, P>(tile, V.R, V.K, tid, nthr);
 }
 
-// By one warp.  Returns the tile's exponent, or -1 for a tile that needs FP64.
+// By one warp.  Returns the tile's exponent (tile_exponent).
 template <int TS, int P, typename T>
 __device__ __forceinline__ int load_fx(int2 *tile, const T *src, int R, int K, int rs, int cs, int lane) {
   const View<TS> V(R, K, rs, cs);
   const TileMax mx = read_raw<TS, P>(tile, src, V, rs, cs, lane, 32);
   const unsigned hi = __reduce_max_sync(kFull, mx.hi), any = __reduce_or_sync(kFull, mx.any);
-  if (tile_special(hi, any)) return -1;
-  const int E = (int)(hi >> 20);
-  raw_to_limbs<TS, P>(tile, V, E, lane, 32);
+  const int E = tile_exponent(hi, any);
+  if (E >= 0) raw_to_limbs<TS, P>(tile, V, E, lane, 32);
   return E;
 }
 
@@ -138,11 +137,10 @@ __device__ __forceinline__ int load_fx_cta(int2 *tile, const T *src, int R, int 
     hi = max(hi, red[2 * w]);
     any |= red[2 * w + 1];
   }
-  const bool bad = tile_special(hi, any);
-  const int E = (int)(hi >> 20);
-  if (!bad) raw_to_limbs<TS, P>(tile, V, E, tid, 32 * WC);
+  const int E = tile_exponent(hi, any);
+  if (E >= 0) raw_to_limbs<TS, P>(tile, V, E, tid, 32 * WC);
   __syncthreads();
-  return bad ? -1 : E;
+  return E;
 }
 
 template <int TS, int P, typename T>
@@ -172,7 +170,9 @@ __device__ __forceinline__ void load_f32(float *tile, const T *src, int R, int K
 
 // One 16-row pass of T (+)= X Y over a chunk of the inner dimension.  While further
 // chunks follow, the sums are kept in the T tile as 64-bit integers in units of 2^eraw;
-// the last chunk normalises them to limbs under the exponent it returns.
+// the last chunk normalises them to limbs under the exponent it returns.  A chunk with a tile
+// of zeros (exponent 0) has an e below that of any other chunk, so that it never moves the sums
+// of the others; sums that are all zero get eraw = 0.
 template <int TS, int P, int NB>
 __device__ __forceinline__ void stage1_fx(const int2 *X, const int2 *Y, int2 *T, int pass, int m, int pc, int kc,
                                           int lane, bool first, bool last, int extra, int e, int &eraw) {
@@ -230,6 +230,10 @@ __device__ __forceinline__ void stage1_fx(const int2 *X, const int2 *Y, int2 *T,
       }
     lo = __reduce_max_sync(kFull, lo);
     bits = 33 - __clz(lo);
+    if (lo == 0) {
+      bits = 57;
+      e = 0;
+    }
   }
   const int sh = bits - 57;
   eraw = e + sh;
@@ -379,7 +383,7 @@ __global__ void __launch_bounds__(WC == 1 ? 256 : 32 * WC, WC == 1 ? (TS == 32 ?
             E1 = xid ? load_fx<TS, P>(T, Y + (int64_t)it.r0 * e.yrs + (int64_t)pt * e.ycs, m, pc, e.yrs, e.ycs, lane)
                      : load_fx<TS, P>(T, X + (int64_t)pt * e.xcs, m, pc, e.xrs, e.xcs, lane);
 #pragma unroll
-          for (int i = 0; i < NP; ++i) eT[i] = E1 - 1079;
+          for (int i = 0; i < NP; ++i) eT[i] = zero_as_one(E1) - 1079;
           slow = E1 < 0;
         } else if (pc > 0) {
           if (both) {
@@ -523,7 +527,7 @@ __global__ void __launch_bounds__(WC == 1 ? 256 : 32 * WC, WC == 1 ? (TS == 32 ?
                 }
               }
             } else {
-              const int e0 = 58 - Shift<TS>::value + Ez - 1079;
+              const int e0 = 58 - Shift<TS>::value + zero_as_one(Ez) - 1079;
               switch (nbq) {
                 case 1:
                   stage2_fx<TS, P, 1, NBMAX, 0>(Tj, Bs, m, kc, lane, scaled(e.f, e0 + eTj[0]), D);

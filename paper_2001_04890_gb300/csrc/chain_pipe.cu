@@ -71,7 +71,7 @@ __device__ __forceinline__ int block_exponent(const T *src, int64_t n, int lane)
   TileMax mx;
   for (int64_t i = lane; i < n; i += 32) mx.add((double)src[i]);
   const unsigned hi = __reduce_max_sync(kFull, mx.hi), any = __reduce_or_sync(kFull, mx.any);
-  return tile_special(hi, any) ? -1 : (int)(hi >> 20);
+  return zero_as_one(tile_exponent(hi, any));
 }
 
 // Images of the operator blocks, one warp per block.
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(128) psi_images_kernel(const PsiSpan *__restri
       hi = max(hi, red[w]);
       any |= red[4 + w];
     }
-    E = tile_special(hi, any) ? -1 : (int)(hi >> 20);
+    E = zero_as_one(tile_exponent(hi, any));
     if (tid == 0) exps[blockIdx.x] = E;
     if (E < 0) return;
   }

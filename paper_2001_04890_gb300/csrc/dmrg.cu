@@ -863,15 +863,38 @@ struct OpSet {
   DBuf<int> id;  // slab of the identity of each dimension, or -1
   int max_id = -1;
   int64_t nblocks = 0;
+  uint64_t need = 0;  // bytes of the images
   bool ready = false, tried = false;
+  void clear() {
+    slabs.clear();
+    nblocks = 0;
+    need = 0;
+  }
+  // K blocks of rows x cols from element address src on (~0: the identity)
+  void add(bool f32, uint64_t src, int rows, int cols, int K) {
+    if (K <= 0 || rows <= 0 || cols <= 0) return;
+    slabs.push_back({src, need, nblocks, rows, cols});
+    nblocks += K;
+    need += (uint64_t)K * (pipe_image_size(f32, rows, cols) + pipe_image_size(f32, cols, rows)) * (f32 ? 4 : 8);
+  }
+  void make(bool f32, cudaStream_t s) {  // the images of what was added
+    images.alloc((size_t)std::max<uint64_t>(need, 1));
+    exps.alloc((size_t)std::max<int64_t>(nblocks, 1));
+    for (OpSlab &x : slabs) x.img += (uint64_t)(uintptr_t)images.p;
+    DBuf<OpSlab> by_block;  // in the order of the blocks, before they are sorted
+    by_block.upload(slabs, s);
+    CK(launch_op_images(by_block.p, (int)slabs.size(), nblocks, exps.p, f32, s));
+    CK(cudaStreamSynchronize(s));
+    upload(s);
+    ready = true;
+  }
   void release() {
     images.release();
     dslabs.release();
     exps.release();
     id.release();
-    slabs.clear();
+    clear();
     max_id = -1;
-    nblocks = 0;
     ready = tried = false;
   }
   size_t bytes() const { return images.n; }
@@ -1573,15 +1596,7 @@ static void build_images(dmrg_ctx *c, bool f32) {
   if (S.tried) return;
   DevBlock *blk[2] = {lblock(c), rblock(c)};
   const uint64_t esize = f32 ? 4 : 8;
-  S.slabs.clear();
-  S.nblocks = 0;
-  uint64_t need = 0;
-  auto slab = [&](uint64_t src, int rows, int cols, int K) {
-    if (K <= 0 || rows <= 0 || cols <= 0) return;
-    S.slabs.push_back({src, need, S.nblocks, rows, cols});
-    S.nblocks += K;
-    need += (uint64_t)K * (pipe_image_size(f32, rows, cols) + pipe_image_size(f32, cols, rows)) * esize;
-  };
+  S.clear();
   const double *src64[4] = {blk[0]->arena(), blk[1]->arena(), P.temps.arena[0].p, P.temps.arena[1].p};
   for (int i = 0; i < 4; ++i) {
     const BlockLayout &b = blk[i & 1]->lay;
@@ -1589,7 +1604,7 @@ static void build_images(dmrg_ctx *c, bool f32) {
     const uint64_t e0 = (uint64_t)(uintptr_t)base / esize;
     auto family = [&](const std::vector<int> &bra, const std::vector<int64_t> &off, int64_t fbase, int K) {
       for (int a = 0; a < (int)b.sec.size(); ++a)
-        if (bra[a] >= 0) slab(e0 + (uint64_t)(fbase + off[a]), b.sec[bra[a]].dim, b.sec[a].dim, K);
+        if (bra[a] >= 0) S.add(f32, e0 + (uint64_t)(fbase + off[a]), b.sec[bra[a]].dim, b.sec[a].dim, K);
     };
     if (i < 2)
       for (const Family &F : b.fam) family(F.bra, F.off, F.base, F.K());
@@ -1600,25 +1615,17 @@ static void build_images(dmrg_ctx *c, bool f32) {
   for (int i = 0; i < 2; ++i)
     for (const Sector &sec : blk[i]->lay.sec) {
       if ((int)has.size() <= sec.dim) has.resize((size_t)sec.dim + 1, 0);
-      if (!has[(size_t)sec.dim]) slab(~0ull, sec.dim, sec.dim, 1);
+      if (!has[(size_t)sec.dim]) S.add(f32, ~0ull, sec.dim, sec.dim, 1);
       has[(size_t)sec.dim] = 1;
     }
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  if (need > (free_b + S.images.n) / 3) {
+  if (S.need > (free_b + S.images.n) / 3) {
     S.release();
     S.tried = true;
     return;
   }
-  S.images.alloc((size_t)std::max<uint64_t>(need, 1));
-  S.exps.alloc((size_t)std::max<int64_t>(S.nblocks, 1));
-  for (OpSlab &x : S.slabs) x.img += (uint64_t)(uintptr_t)S.images.p;
-  DBuf<OpSlab> by_block;  // in the order of the blocks, before they are sorted
-  by_block.upload(S.slabs, c->stream);
-  CK(launch_op_images(by_block.p, (int)S.slabs.size(), S.nblocks, S.exps.p, f32, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  S.upload(c->stream);
-  S.ready = true;
+  S.make(f32, c->stream);
   S.tried = true;
 }
 
@@ -3451,6 +3458,77 @@ extern "C" int dmrg_selftest_tcgen05(int N, int K, const float *A, const float *
   CK(cudaMemcpy(&status, st.p, sizeof(int), cudaMemcpyDeviceToHost));
   CK(cudaMemcpy(C, cc.p, (size_t)128 * N * sizeof(float), cudaMemcpyDeviceToHost));
   if (status) throw Fail{DMRG_ETIMEOUT, "tcgen05 self-test: mbarrier wait ran out"};
+  API_END
+}
+
+// D = sum_t f_t X_t Y Z_t for one output block through the kernels that the task lists run on.
+extern "C" int dmrg_selftest_chain(int kind, int ntasks, int m, int n, int p, int q, const double *X, const double *Y,
+                                   const double *Z, const double *f, double *D) {
+  API_BEGIN
+  const int big = 1024;
+  if (kind < 0 || kind > 3 || ntasks < 1 || ntasks > 4096 || m < 1 || n < 1 || p < 1 || q < 1 || m > big || n > big ||
+      p > big || q > big || !Y || !f || !D || (!X && n != m) || (!Z && p != q))
+    throw Fail{DMRG_EINVAL, "dmrg_selftest_chain: kind 0..3, 1..4096 tasks, sides 1..1024; an identity is square"};
+  const bool f32 = kind >= 2, prepared = kind % 2 == 0;
+  cudaStream_t s = nullptr;
+  const size_t nx = (size_t)m * n, nz = (size_t)p * q;
+  if ((nx + nz) * ntasks > (size_t(1) << 24)) throw Fail{DMRG_EINVAL, "dmrg_selftest_chain: 2^24 operator elements at most"};
+  DBuf<double> x, y, z, d;
+  DBuf<float> x32, z32;
+  auto take = [&](DBuf<double> &b, const double *h, size_t count) {
+    b.alloc(count);
+    CK(cudaMemcpyAsync(b.p, h, count * sizeof(double), cudaMemcpyHostToDevice, s));
+  };
+  auto address = [&](const double *h, DBuf<double> &b, DBuf<float> &b32, size_t count) -> uint64_t {
+    if (!h) return ~0ull;
+    take(b, h, count);
+    if (!f32) return eaddr(b.p);
+    b32.alloc(count);
+    CK(launch_to_f32(b32.p, b.p, (int64_t)count, s));
+    return (uint64_t)(uintptr_t)b32.p / 4;
+  };
+  const uint64_t xa = address(X, x, x32, nx * ntasks), za = address(Z, z, z32, nz * ntasks);
+  take(y, Y, (size_t)n * p);
+  d.alloc((size_t)m * q);
+  CK(cudaMemsetAsync(d.p, 0, (size_t)m * q * sizeof(double), s));
+  ChainList CL;
+  for (int t = 0; t < ntasks; ++t) {
+    ChainEntry e{};
+    e.x = X ? xa + t * nx : ~0ull;
+    e.xrs = X ? n : 0;
+    e.xcs = X ? 1 : 0;
+    e.y = 0;
+    e.yrs = p;
+    e.ycs = 1;
+    e.z = Z ? za + t * nz : ~0ull;
+    e.zrs = Z ? q : 0;
+    e.zcs = Z ? 1 : 0;
+    e.n = n;
+    e.p = p;
+    e.f = f[t];
+    CL.ent.push_back({0, e});
+  }
+  ChainGroup g{};
+  g.drs = q;
+  g.dcs = 1;
+  g.m = m;
+  g.q = q;
+  CL.finish({g});
+  DevChain ch;
+  ch.upload(CL, s, false, false, ChainTune(), f32);
+  OpSet ops;
+  if (prepared) {
+    if (X) ops.add(f32, xa, m, n, ntasks);
+    if (Z) ops.add(f32, za, p, q, ntasks);
+    if (!X) ops.add(f32, ~0ull, m, m, 1);
+    if (!Z && (X || m != q)) ops.add(f32, ~0ull, q, q, 1);
+    ops.make(f32, s);
+    ch.prepare(&ops, {PsiSpan{0, 0, n, p}}, s);
+    if (!ch.pipe) throw Fail{DMRG_EINVAL, "dmrg_selftest_chain: the prepared kernels do not take this shape"};
+  }
+  ch.launch(0, (uint64_t)(uintptr_t)y.p, 0, (uint64_t)(uintptr_t)d.p, s);
+  CK(cudaMemcpyAsync(D, d.p, (size_t)m * q * sizeof(double), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
   API_END
 }
 
