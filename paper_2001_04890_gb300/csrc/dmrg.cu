@@ -89,7 +89,9 @@ static cudaError_t device_alloc(void **p, size_t bytes) {
       break;
     }
   }
-  return cudaMalloc(p, bytes);
+  const cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, not by the next launch's check
+  return e;
 }
 
 template <class T>
@@ -877,7 +879,19 @@ struct OpSet {
     nblocks += K;
     need += (uint64_t)K * (pipe_image_size(f32, rows, cols) + pipe_image_size(f32, cols, rows)) * (f32 ? 4 : 8);
   }
-  void make(bool f32, cudaStream_t s) {  // the images of what was added
+  // The images of what was added; without memory for them there are none (ready stays false), and
+  // the general kernels convert as they read.
+  void make(bool f32, cudaStream_t s) {
+    try {
+      build(f32, s);
+      ready = true;
+    } catch (const Fail &e) {
+      if (e.code != DMRG_ENOMEM) throw;
+      CK(cudaStreamSynchronize(s));
+      release();
+    }
+  }
+  void build(bool f32, cudaStream_t s) {
     images.alloc((size_t)std::max<uint64_t>(need, 1));
     exps.alloc((size_t)std::max<int64_t>(nblocks, 1));
     for (OpSlab &x : slabs) x.img += (uint64_t)(uintptr_t)images.p;
@@ -886,7 +900,6 @@ struct OpSet {
     CK(launch_op_images(by_block.p, (int)slabs.size(), nblocks, exps.p, f32, s));
     CK(cudaStreamSynchronize(s));
     upload(s);
-    ready = true;
   }
   void release() {
     images.release();
@@ -993,7 +1006,7 @@ struct DevChain {
   DBuf<uint8_t> pimages;
   int nspans = 0;
   SideStreams side;  // for the kernels of several classes
-  bool forked() const { return pipe && side.s[0]; }
+  bool forked() const { return pipe && side.ev[2]; }
   bool on_cores() const {
     for (int n : nitems)
       if (n > 0) return true;
@@ -1001,11 +1014,32 @@ struct DevChain {
   }
 
   // Run the list's CUDA-core chunks on prepared operands: o over the list's own operators, sp
-  // the psi blocks.
+  // the psi blocks.  Where they do not take the list, or memory for them is short, the general
+  // kernels run it.
   void prepare(const OpSet *o, std::vector<PsiSpan> sp, cudaStream_t s) {
     pipe = false;
     ops = o;
-    if (!on_cores() || !o || !o->ready || sp.size() >= (size_t(1) << 24)) return;
+    if (on_cores() && o && o->ready && sp.size() < (size_t(1) << 24)) {
+      try {
+        build_entries(o, sp, s);
+      } catch (const Fail &e) {
+        pipe = false;
+        if (e.code != DMRG_ENOMEM) throw;
+        CK(cudaStreamSynchronize(s));
+      }
+    }
+    if (!pipe) release_prepared();
+  }
+  void release_prepared() {
+    pent.release();
+    stacks.release();
+    nstacks.release();
+    spans.release();
+    pexp.release();
+    pimages.release();
+    pipe = false;
+  }
+  void build_entries(const OpSet *o, std::vector<PsiSpan> &sp, cudaStream_t s) {
     int64_t img = 0;
     for (PsiSpan &b : sp) {
       b.img = img;
@@ -1026,10 +1060,10 @@ struct DevChain {
     int is_bad = 0;
     CK(cudaMemcpyAsync(&is_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));  // also: sp may be released
-    pipe = !is_bad;                // else the general kernels take the list
     int kernels = ntc > 0 ? 1 : 0;
     for (int n : nitems) kernels += n > 0;
-    if (pipe && kernels > 1) side.create();
+    if (!is_bad && kernels > 1) side.create();
+    pipe = !is_bad;
   }
 
   void upload(const ChainList &CL, cudaStream_t s, bool tensor_cores = false, bool split_tasks = false,
@@ -1132,13 +1166,7 @@ struct DevChain {
     all.release();
     cores.release();
     items.release();
-    pent.release();
-    stacks.release();
-    nstacks.release();
-    spans.release();
-    pexp.release();
-    pimages.release();
-    pipe = false;
+    release_prepared();
     ops = nullptr;
     red.release();
     scratch.release();
@@ -1622,10 +1650,9 @@ static void build_images(dmrg_ctx *c, bool f32) {
   CK(cudaMemGetInfo(&free_b, &total_b));
   if (S.need > (free_b + S.images.n) / 3) {
     S.release();
-    S.tried = true;
-    return;
+  } else {
+    S.make(f32, c->stream);
   }
-  S.make(f32, c->stream);
   S.tried = true;
 }
 
@@ -3523,6 +3550,7 @@ extern "C" int dmrg_selftest_chain(int kind, int ntasks, int m, int n, int p, in
     if (!X) ops.add(f32, ~0ull, m, m, 1);
     if (!Z && (X || m != q)) ops.add(f32, ~0ull, q, q, 1);
     ops.make(f32, s);
+    if (!ops.ready) throw Fail{DMRG_ENOMEM, "dmrg_selftest_chain: no memory for the operand images"};
     ch.prepare(&ops, {PsiSpan{0, 0, n, p}}, s);
     if (!ch.pipe) throw Fail{DMRG_EINVAL, "dmrg_selftest_chain: the prepared kernels do not take this shape"};
   }
