@@ -60,7 +60,11 @@ enum {
  * FP64 operators (no FP32 copies are held), and the remaining blocks run in
  * FP64.  In both mixed modes Davidson finishes with a defect-corrected
  * refinement that applies H in FP64 to the current vector (see dmrg_davidson),
- * so energies are FP64 quality. */
+ * so energies are FP64 quality.
+ * Device memory: for H.psi in FP64 or FP32 a context keeps its position's operators in prepared
+ * form beside them (4 to 20 times their bytes, the more the smaller the blocks) if that takes at
+ * most a third of the free memory.  They are given back when an allocation of one of the
+ * context's calls fails; H.psi then runs without them until the position is planned again. */
 enum { DMRG_PREC_FP64 = 0, DMRG_PREC_FP32 = 1, DMRG_PREC_BF16X3 = 2 };
 
 typedef struct dmrg_ctx dmrg_ctx; /* opaque, library-owned */

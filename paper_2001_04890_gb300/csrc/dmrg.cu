@@ -94,6 +94,22 @@ static cudaError_t device_alloc(void **p, size_t bytes) {
   return e;
 }
 
+// The contexts of the call that runs on this thread.  Their operator images are an option: an
+// allocation of the call that fails gives them back (the general kernels run from then on) and is
+// tried once more.
+struct GivesBack {
+  static thread_local const GivesBack *top;
+  const GivesBack *outer;
+  dmrg_ctx *const *ctx;
+  int n;
+  GivesBack(dmrg_ctx *const *ctx, int n) : outer(top), ctx(ctx), n(n) { top = this; }
+  ~GivesBack() { top = outer; }
+  GivesBack(const GivesBack &) = delete;
+  GivesBack &operator=(const GivesBack &) = delete;
+};
+thread_local const GivesBack *GivesBack::top = nullptr;
+static bool give_back_images();  // whether there were any
+
 template <class T>
 struct DBuf {
   T *p = nullptr;
@@ -111,7 +127,10 @@ struct DBuf {
     if (count <= n && p) return;
     release();
     if (count == 0) return;
-    CK(device_alloc(reinterpret_cast<void **>(&p), count * sizeof(T)));
+    cudaError_t cudaMalloc_result = device_alloc(reinterpret_cast<void **>(&p), count * sizeof(T));
+    if (cudaMalloc_result == cudaErrorMemoryAllocation && give_back_images())
+      cudaMalloc_result = device_alloc(reinterpret_cast<void **>(&p), count * sizeof(T));
+    CK(cudaMalloc_result);
     n = count;
   }
   template <class A>
@@ -858,7 +877,7 @@ static constexpr size_t kImagesKept = size_t(1) << 30;
 // The operators of a position as images (chain_pipe.cu): digits of the FP64 operators and
 // temporaries, or their FP32 copies.
 struct OpSet {
-  DBuf<uint8_t> images;
+  std::shared_ptr<DBuf<uint8_t>> images;  // a batch over the context holds them too
   std::vector<OpSlab> slabs;  // sorted by src once uploaded
   DBuf<OpSlab> dslabs;
   DBuf<int16_t> exps;
@@ -882,6 +901,7 @@ struct OpSet {
   // The images of what was added; without memory for them there are none (ready stays false), and
   // the general kernels convert as they read.
   void make(bool f32, cudaStream_t s) {
+    const GivesBack none(nullptr, 0);
     try {
       build(f32, s);
       ready = true;
@@ -892,9 +912,13 @@ struct OpSet {
     }
   }
   void build(bool f32, cudaStream_t s) {
-    images.alloc((size_t)std::max<uint64_t>(need, 1));
+    if (!images || images->n < need) {
+      images.reset();
+      images = std::make_shared<DBuf<uint8_t>>();
+      images->alloc((size_t)std::max<uint64_t>(need, 1));
+    }
     exps.alloc((size_t)std::max<int64_t>(nblocks, 1));
-    for (OpSlab &x : slabs) x.img += (uint64_t)(uintptr_t)images.p;
+    for (OpSlab &x : slabs) x.img += (uint64_t)(uintptr_t)images->p;
     DBuf<OpSlab> by_block;  // in the order of the blocks, before they are sorted
     by_block.upload(slabs, s);
     CK(launch_op_images(by_block.p, (int)slabs.size(), nblocks, exps.p, f32, s));
@@ -902,7 +926,7 @@ struct OpSet {
     upload(s);
   }
   void release() {
-    images.release();
+    images.reset();
     dslabs.release();
     exps.release();
     id.release();
@@ -910,7 +934,7 @@ struct OpSet {
     max_id = -1;
     ready = tried = false;
   }
-  size_t bytes() const { return images.n; }
+  size_t bytes() const { return images ? images->n : 0; }
   OpTable table() const { return {dslabs.p, exps.p, id.p, (int)slabs.size(), max_id}; }
   // the slabs to the device, sorted by source; the identities (src ~0) come last
   void upload(cudaStream_t s) {
@@ -1020,6 +1044,7 @@ struct DevChain {
     pipe = false;
     ops = o;
     if (on_cores() && o && o->ready && sp.size() < (size_t(1) << 24)) {
+      const GivesBack none(nullptr, 0);
       try {
         build_entries(o, sp, s);
       } catch (const Fail &e) {
@@ -1324,6 +1349,7 @@ struct HPlan {
   DBuf<float> f32[4];  // left ops, right ops, left temps, right temps
   OpSet ops32;         // images of them
   DevChain chain32;
+  bool captured = false;  // a caller's graph reads the images and list entries
 };
 
 }  // namespace dmrg
@@ -1368,6 +1394,27 @@ struct dmrg_ctx {
 };
 
 namespace dmrg {
+
+static bool give_back_images() {
+  bool any = false;
+  if (!GivesBack::top) return false;
+  for (int i = 0; i < GivesBack::top->n; ++i) {
+    dmrg_ctx *c = GivesBack::top->ctx[i];
+    if (!c || c->plan.captured) continue;
+    HPlan &P = c->plan;
+    for (OpSet *S : {&P.ops, &P.ops32}) {
+      if (!S->bytes()) continue;
+      CK(cudaStreamSynchronize(c->stream));
+      for (DevChain *ch : {&P.chain, &P.chain32})
+        if (ch->ops == S) ch->release_prepared();
+      const bool tried = S->tried;
+      S->release();
+      S->tried = tried;
+      any = true;
+    }
+  }
+  return any;
+}
 
 static DevBlock *lblock(dmrg_ctx *c) {
   return c->k < (int)c->left.size() ? c->left[c->k].get() : nullptr;
@@ -1648,7 +1695,7 @@ static void build_images(dmrg_ctx *c, bool f32) {
     }
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  if (S.need > (free_b + S.images.n) / 3) {
+  if (S.need > (free_b + S.bytes()) / 3) {
     S.release();
   } else {
     S.make(f32, c->stream);
@@ -1677,6 +1724,7 @@ static void build_hplan(dmrg_ctx *c) {
   P.psi = psi_layout(lb->lay, rb->lay, c->nu, c->nd);
   const Psi &Y = P.psi;
   P.temps.set = TempSet();
+  P.captured = false;
   P.ops.ready = P.ops.tried = P.ops32.ready = P.ops32.tried = false;
   P.chain.pipe = P.chain32.pipe = false;
   P.chain.ops = P.chain32.ops = nullptr;
@@ -2866,6 +2914,7 @@ extern "C" int dmrg_enlarged_layout(dmrg_ctx *c, int direction, int *nsec, int *
 
 extern "C" int dmrg_hpsi(dmrg_ctx *c, const double *psi, double *sigma, int device_ptrs) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || !psi || !sigma) throw Fail{DMRG_EINVAL, "NULL argument"};
   build_hplan(c);
   const int64_t n = c->plan.psi.dim;
@@ -2886,6 +2935,7 @@ extern "C" int dmrg_hpsi(dmrg_ctx *c, const double *psi, double *sigma, int devi
 
 extern "C" int dmrg_hpsi_flops(dmrg_ctx *c, double *flops, long long *tasks) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c) throw Fail{DMRG_EINVAL, "ctx is NULL"};
   build_hplan(c);
   if (flops) *flops = c->plan.flops;
@@ -2895,6 +2945,7 @@ extern "C" int dmrg_hpsi_flops(dmrg_ctx *c, double *flops, long long *tasks) {
 
 extern "C" int dmrg_set_psi(dmrg_ctx *c, const double *psi, int device_ptr) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || !psi) throw Fail{DMRG_EINVAL, "NULL argument"};
   build_hplan(c);
   const int64_t n = c->plan.psi.dim;
@@ -2908,6 +2959,7 @@ extern "C" int dmrg_set_psi(dmrg_ctx *c, const double *psi, int device_ptr) {
 
 extern "C" int dmrg_get_psi(dmrg_ctx *c, double *psi, int device_ptr) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || !psi) throw Fail{DMRG_EINVAL, "NULL argument"};
   if (!c->psi_valid) throw Fail{DMRG_ESTATE, "no wave function at this position"};
   build_hplan(c);
@@ -2919,6 +2971,7 @@ extern "C" int dmrg_get_psi(dmrg_ctx *c, double *psi, int device_ptr) {
 
 extern "C" int dmrg_davidson(dmrg_ctx *c, double tol, int max_iter, double *energy, int *iters) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || !(tol > 0.0) || max_iter < 1) throw Fail{DMRG_EINVAL, "bad arguments"};
   bool conv = false;
   davidson(c, tol, max_iter, energy, iters, conv);
@@ -2929,6 +2982,7 @@ extern "C" int dmrg_davidson(dmrg_ctx *c, double tol, int max_iter, double *ener
 
 extern "C" int dmrg_davidson_lowp(dmrg_ctx *c, double tol, int max_iter, double *energy, int *iters) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || !(tol > 0.0) || max_iter < 1) throw Fail{DMRG_EINVAL, "bad arguments"};
   build_hplan(c);
   bool conv = false;
@@ -2945,6 +2999,7 @@ extern "C" int dmrg_renormalize(dmrg_ctx *c, int direction, const int *kept, con
                                 double *discarded_weight) {
   API_BEGIN
   if (!c || (direction != 1 && direction != -1)) throw Fail{DMRG_EINVAL, "bad arguments"};
+  const GivesBack images(&c, 1);
   do_renormalize(c, direction, O ? kept : nullptr, O, discarded_weight, O ? nullptr : const_cast<int *>(kept));
   API_END
 }
@@ -2981,6 +3036,7 @@ static void sweep_impl(dmrg_ctx *c, int nsweeps, double tol, double *energies, d
 
 extern "C" int dmrg_sweep(dmrg_ctx *c, int nsweeps, double tol, double *energies) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || nsweeps < 0 || !(tol > 0.0)) throw Fail{DMRG_EINVAL, "bad arguments"};
   if (c->L < 3) throw Fail{DMRG_EINVAL, "sweeps need L >= 3"};
   sweep_impl(c, nsweeps, tol, energies, nullptr, nullptr);
@@ -2992,6 +3048,7 @@ extern "C" int dmrg_sweep_record(dmrg_ctx *c, int nsweeps, double tol, double *e
   API_BEGIN
   if (!c || nsweeps < 0 || !(tol > 0.0)) throw Fail{DMRG_EINVAL, "bad arguments"};
   if (c->L < 3) throw Fail{DMRG_EINVAL, "sweeps need L >= 3"};
+  const GivesBack images(&c, 1);
   sweep_impl(c, nsweeps, tol, energies, discarded, entropies);
   API_END
 }
@@ -3630,6 +3687,11 @@ extern "C" int dmrg_hpsi_noalloc(dmrg_ctx *c, const double *psi, double *sigma) 
                                 " doubles of H.psi scratch; the no-allocation scratch holds " +
                                 std::to_string(kNoAllocScratchDoubles) + " (use dmrg_hpsi)"};
   double *scratch = noalloc_scratch();
+  if (c->stream) {  // captured: what the graph reads stays until the list is rebuilt
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(c->stream, &st));
+    if (st != cudaStreamCaptureStatusNone) P.captured = true;
+  }
   // a time-out left by an earlier call is not this call's: clear the status word
   // (a time-out of this call is read by dmrg_check_status or the next synchronizing call)
   CK(cudaMemsetAsync(c->dstatus.p, 0, 8 * sizeof(int), c->stream));
@@ -3654,7 +3716,8 @@ struct dmrg_batch {
   dmrg::ChainTune tune;
   DevChain chain;
   DBuf<double> psi, sigma;
-  OpSet ops;  // tables over the contexts' operator images (the images stay theirs)
+  OpSet ops;  // tables over the contexts' operator images
+  std::vector<std::shared_ptr<DBuf<uint8_t>>> images;
   std::vector<PsiSpan> spans;
   double flops = 0.0;
   cudaGraph_t graph = nullptr;
@@ -3703,10 +3766,13 @@ static void batch_chainlist(const std::vector<dmrg_ctx *> &ctxs, ChainList &CL, 
   }
 }
 
-// The contexts' operator images as one set.
+// The contexts' operator images as one set, which stay with the batch when a context gives its
+// own back.
 static void batch_images(dmrg_batch *b, cudaStream_t s) {
+  const GivesBack none(nullptr, 0);
   OpSet &S = b->ops;
   S.release();
+  b->images.clear();
   const bool f32 = b->ctx[0]->prec == DMRG_PREC_FP32;
   for (dmrg_ctx *c : b->ctx) {
     if ((c->prec == DMRG_PREC_FP32) != f32) return;
@@ -3715,19 +3781,27 @@ static void batch_images(dmrg_batch *b, cudaStream_t s) {
     if (!L.ready) return;  // memory: the batch converts as it reads
     S.nblocks += L.nblocks;
   }
-  S.exps.alloc((size_t)std::max<int64_t>(S.nblocks, 1));
-  int64_t first = 0;
-  for (dmrg_ctx *c : b->ctx) {
-    const OpSet &L = f32 ? c->plan.ops32 : c->plan.ops;
-    for (OpSlab x : L.slabs) {
-      x.first += first;
-      S.slabs.push_back(x);
+  try {
+    S.exps.alloc((size_t)std::max<int64_t>(S.nblocks, 1));
+    int64_t first = 0;
+    for (dmrg_ctx *c : b->ctx) {
+      const OpSet &L = f32 ? c->plan.ops32 : c->plan.ops;
+      for (OpSlab x : L.slabs) {
+        x.first += first;
+        S.slabs.push_back(x);
+      }
+      CK(cudaMemcpyAsync(S.exps.p + first, L.exps.p, L.nblocks * sizeof(int16_t), cudaMemcpyDeviceToDevice, s));
+      first += L.nblocks;
+      b->images.push_back(L.images);
     }
-    CK(cudaMemcpyAsync(S.exps.p + first, L.exps.p, L.nblocks * sizeof(int16_t), cudaMemcpyDeviceToDevice, s));
-    first += L.nblocks;
+    S.upload(s);
+    S.ready = true;
+  } catch (const Fail &e) {
+    if (e.code != DMRG_ENOMEM) throw;
+    CK(cudaStreamSynchronize(s));
+    S.release();
+    b->images.clear();
   }
-  S.upload(s);
-  S.ready = true;
 }
 
 extern "C" int dmrg_batch_create(int n, dmrg_ctx *const *ctxs, dmrg_batch **out) {
@@ -3744,6 +3818,7 @@ extern "C" int dmrg_batch_create(int n, dmrg_ctx *const *ctxs, dmrg_batch **out)
       throw Fail{DMRG_EINVAL, "batched contexts must share the working precision class"};
     b->ctx.push_back(c);
   }
+  const GivesBack images(ctxs, n);
   ChainList CL;
   batch_chainlist(b->ctx, CL, b->off, b->flops);
   for (dmrg_ctx *c : b->ctx) b->gen.push_back(c->plan_gen);
@@ -3935,6 +4010,7 @@ static void tune_out(const ChainTune &t, double *params) {
 
 extern "C" int dmrg_autotune(dmrg_ctx *c, int reps, double *best_ms, double *params) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || reps < 1) throw Fail{DMRG_EINVAL, "dmrg_autotune: NULL context or reps < 1"};
   build_hplan(c);
   HPlan &P = c->plan;
@@ -4262,6 +4338,7 @@ static void mutual_information(dmrg_ctx *c, double *I, double *s1, double *rho_a
 
 extern "C" int dmrg_mutual_information(dmrg_ctx *c, double *I, double *s1, double *rho_pairs) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || (!I && !s1 && !rho_pairs)) throw Fail{DMRG_EINVAL, "NULL argument"};
   if (c->L < 2) throw Fail{DMRG_EINVAL, "mutual information needs L >= 2"};
   mutual_information(c, I, s1, rho_pairs);
@@ -4270,6 +4347,7 @@ extern "C" int dmrg_mutual_information(dmrg_ctx *c, double *I, double *s1, doubl
 
 extern "C" int dmrg_orbital_entropies(dmrg_ctx *c, double *s3, double *rho2) {
   API_BEGIN
+  const GivesBack images(&c, 1);
   if (!c || (!s3 && !rho2)) throw Fail{DMRG_EINVAL, "NULL argument"};
   current_entropies(c, s3, rho2);
   API_END
@@ -4286,27 +4364,31 @@ extern "C" int dmrg_batch_autotune(dmrg_batch *b, int reps, double *best_ms, dou
   API_BEGIN
   if (!b || reps < 1) throw Fail{DMRG_EINVAL, "dmrg_batch_autotune: NULL batch or reps < 1"};
   CK(cudaStreamSynchronize(b->stream));
+  const GivesBack images(b->ctx.data(), (int)b->ctx.size());
   ChainList CL;
   std::vector<long long> off;
   double fl = 0.0;
   batch_chainlist(b->ctx, CL, off, fl);
   if (off != b->off) throw Fail{DMRG_ESTATE, "a batched context changed position since dmrg_batch_create"};
-  b->gen.clear();
-  for (dmrg_ctx *c : b->ctx) b->gen.push_back(c->plan_gen);
+  // the batch keeps what its present list reads until it builds the new one
+  std::vector<long long> gen;
+  for (dmrg_ctx *c : b->ctx) gen.push_back(c->plan_gen);
   const int64_t n = b->off.back();
-  batch_images(b, b->stream);
+  if (gen != b->gen || !b->ops.ready) batch_images(b, b->stream);
   CK(launch_fill_guess(b->psi.p, n, 0x5eedull, b->stream));
   double ms = 0.0;
   ChainTune best = autotune_chain(CL, b->tc, b->ctx[0]->prec == DMRG_PREC_FP32, b->psi.p, b->sigma.p, n, b->stream,
                                   b->ctx[0]->dstatus.p, reps, b->tune, ms, &b->ops, b->spans);
   check_status(b->ctx[0]);
-  b->tune = best;
-  b->chain.upload(CL, b->stream, b->tc, true, best, b->ctx[0]->prec == DMRG_PREC_FP32);
-  b->chain.prepare(&b->ops, b->spans, b->stream);
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   b->exec = nullptr;
   b->graph = nullptr;  // captured again on the next dmrg_batch_hpsi
+  b->gen.assign(gen.size(), -1);  // refused from here to the end of the rebuild
+  b->tune = best;
+  b->chain.upload(CL, b->stream, b->tc, true, best, b->ctx[0]->prec == DMRG_PREC_FP32);
+  b->chain.prepare(&b->ops, b->spans, b->stream);
+  b->gen.swap(gen);
   CK(cudaStreamSynchronize(b->stream));
   if (best_ms) *best_ms = ms;
   tune_out(best, params);

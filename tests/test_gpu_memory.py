@@ -63,3 +63,99 @@ def test_every_allocation_of_the_plan_may_fail(prec):
         if untouched >= 12:
             break  # past the last allocation
     assert general >= 6  # images, exponents, slabs, identities; psi spans and images, entries, stacks
+
+
+def _failing(call):
+    """The call with its first device allocation failing."""
+    binding.debug_fail_alloc(1)
+    try:
+        return call()
+    finally:
+        binding.debug_fail_alloc(0)
+
+
+@pytest.mark.parametrize("prec", [binding.PREC_FP64, binding.PREC_FP32, binding.PREC_BF16X3])
+def test_images_are_given_back_when_a_call_needs_the_memory(prec):
+    """The calls after H.psi allocate beside the images: one failure takes those, not the call."""
+    ctx = _context(prec)
+    x = workloads.gaussian(ctx.psi_layout()[1], seed=3)
+    calls = {"hpsi": lambda c: c.hpsi(x), "set_psi": lambda c: (c.set_psi(x), c.get_psi())[1],
+             "davidson": lambda c: (c.set_psi(x), c.davidson(1e-9, 400)[0])[1]}
+    ref, whole = ctx.hpsi(x), _launches(ctx, x)
+    energy = calls["davidson"](ctx)
+    ctx.close()
+    for name, call in calls.items():
+        c = _context(prec)
+        c.hpsi(x)
+        if name == "davidson":
+            c.set_psi(x)
+        y = _failing(lambda: call(c))
+        assert np.max(np.abs(y - {"hpsi": ref, "set_psi": x, "davidson": energy}[name])) <= TOL[prec] * np.max(np.abs(ref)), name
+        assert np.max(np.abs(c.hpsi(x) - ref)) <= TOL[prec] * np.max(np.abs(ref))
+        assert _launches(c, x) < whole  # the general kernels
+        c.set_position(2, 1)
+        c.set_position(3, 1)  # planned again, with images
+        c.hpsi(x)
+        assert _launches(c, x) == whole
+        c.close()
+
+
+def test_renormalization_gives_images_back():
+    ctx = _context(binding.PREC_FP64)
+    x = workloads.gaussian(ctx.psi_layout()[1], seed=3)
+    rng = np.random.default_rng(5)
+    kept = [min(int(d), 6) for _, _, d in ctx.enlarged_layout(1)]
+    O = np.concatenate([workloads.orthonormal_columns(int(d), m, rng).ravel()
+                        for (_, _, d), m in zip(ctx.enlarged_layout(1), kept)])
+    out = []
+    for fail in (False, True):
+        c = _context(binding.PREC_FP64)
+        c.hpsi(x)
+        (_failing if fail else lambda f: f())(lambda: c.renormalize(1, O, kept))
+        out.append(c.hpsi(workloads.gaussian(c.psi_layout()[1], seed=4)))
+        c.close()
+    ctx.close()
+    assert np.array_equal(out[0], out[1])
+
+
+def test_a_batch_keeps_its_contexts_images():
+    ctx = _context(binding.PREC_FP64)
+    x = workloads.gaussian(ctx.psi_layout()[1], seed=3)
+    batch = binding.Batch([ctx])
+    y = batch.hpsi(x)
+    whole = _launches(ctx, x)
+    _failing(lambda: ctx.hpsi(x))
+    assert _launches(ctx, x) < whole
+    assert np.array_equal(batch.hpsi(x), y) and np.array_equal(batch.hpsi(x), y)
+    batch.autotune(reps=1)
+    assert np.max(np.abs(batch.hpsi(x) - y)) <= 1e-12 * np.max(np.abs(y))
+    batch.close()
+    ctx.close()
+
+
+def test_a_captured_call_keeps_its_images():
+    """A graph of dmrg_hpsi_noalloc outlives the call: its images are not given back under it."""
+    import torch
+    stream = torch.cuda.Stream()
+    h, v = workloads.integrals(L, seed=1)
+    ctx = binding.DMRG(h, v, L, 0, M, stream=stream.cuda_stream)
+    workloads.grow_middle_bond(ctx, L, L // 2, L // 2, M, 3, seed=1)
+    x = workloads.gaussian(ctx.psi_layout()[1], seed=3)
+    ref = ctx.hpsi(x)
+    with torch.cuda.stream(stream):
+        psi = torch.from_numpy(x).cuda()
+        sigma = torch.empty_like(psi)
+        ctx.hpsi_noalloc(psi, sigma)
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        ctx.hpsi_noalloc(psi, sigma)
+    with pytest.raises(binding.DMRGError) as err:
+        _failing(lambda: ctx.hpsi(x))
+    assert err.value.code == binding.DMRG_ENOMEM
+    sigma.zero_()
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(sigma.cpu().numpy(), ref)
+    ctx.close()
