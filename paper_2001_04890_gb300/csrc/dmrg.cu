@@ -1662,13 +1662,11 @@ static std::vector<PsiSpan> psi_spans(const Psi &Y, int64_t shift = 0) {
   return v;
 }
 
-// Images of the position's operators and temporaries (f32: of their FP32 copies), unless they
-// would take more than a third of the free device memory (the general kernels then convert as
-// they read).
-static void build_images(dmrg_ctx *c, bool f32) {
+// What has images: the position's operators and temporaries (f32: their FP32 copies) and the
+// identities.
+static void list_images(dmrg_ctx *c, bool f32) {
   HPlan &P = c->plan;
   OpSet &S = f32 ? P.ops32 : P.ops;
-  if (S.tried) return;
   DevBlock *blk[2] = {lblock(c), rblock(c)};
   const uint64_t esize = f32 ? 4 : 8;
   S.clear();
@@ -1693,13 +1691,22 @@ static void build_images(dmrg_ctx *c, bool f32) {
       if (!has[(size_t)sec.dim]) S.add(f32, ~0ull, sec.dim, sec.dim, 1);
       has[(size_t)sec.dim] = 1;
     }
+}
+
+static size_t free_memory() {
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  if (S.need > (free_b + S.bytes()) / 3) {
-    S.release();
-  } else {
-    S.make(f32, c->stream);
-  }
+  return free_b;
+}
+
+// Images of the position, unless they would take more than a third of the free device memory (the
+// general kernels then convert as they read).
+static void build_images(dmrg_ctx *c, bool f32) {
+  OpSet &S = f32 ? c->plan.ops32 : c->plan.ops;
+  if (S.tried) return;
+  list_images(c, f32);
+  if (S.need > (free_memory() + S.bytes()) / 3) S.release();
+  else S.make(f32, c->stream);
   S.tried = true;
 }
 
@@ -3774,8 +3781,16 @@ static void batch_images(dmrg_batch *b, cudaStream_t s) {
   S.release();
   b->images.clear();
   const bool f32 = b->ctx[0]->prec == DMRG_PREC_FP32;
+  uint64_t need = 0;  // of the contexts that have none yet: a third of the free memory for all of them
   for (dmrg_ctx *c : b->ctx) {
     if ((c->prec == DMRG_PREC_FP32) != f32) return;
+    OpSet &L = f32 ? c->plan.ops32 : c->plan.ops;
+    if (L.tried) continue;
+    list_images(c, f32);
+    need += L.need - std::min<uint64_t>(L.need, L.bytes());
+  }
+  if (need > free_memory() / 3) return;
+  for (dmrg_ctx *c : b->ctx) {
     build_images(c, f32);
     const OpSet &L = f32 ? c->plan.ops32 : c->plan.ops;
     if (!L.ready) return;  // memory: the batch converts as it reads
@@ -3829,10 +3844,10 @@ extern "C" int dmrg_batch_create(int n, dmrg_ctx *const *ctxs, dmrg_batch **out)
     const auto sp = psi_spans(b->ctx[i]->plan.psi, b->off[i]);
     b->spans.insert(b->spans.end(), sp.begin(), sp.end());
   }
-  if (b->chain.on_cores()) batch_images(b.get(), b->stream);
-  b->chain.prepare(&b->ops, b->spans, b->stream);
   b->psi.alloc((size_t)std::max<long long>(b->off.back(), 1));
   b->sigma.alloc((size_t)std::max<long long>(b->off.back(), 1));
+  if (b->chain.on_cores()) batch_images(b.get(), b->stream);
+  b->chain.prepare(&b->ops, b->spans, b->stream);
   CK(cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming));

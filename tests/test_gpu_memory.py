@@ -159,3 +159,44 @@ def test_a_captured_call_keeps_its_images():
     torch.cuda.synchronize()
     assert np.array_equal(sigma.cpu().numpy(), ref)
     ctx.close()
+
+
+def test_a_batch_takes_a_third_of_the_free_memory_for_images():
+    """Not a third of what the members before left.  The rest of the device is filled for the second batch."""
+    import torch
+    h, v = workloads.integrals(16, seed=0)
+
+    def members():
+        out = []
+        for n in range(4):
+            c = binding.DMRG(h, v, 16, 0, 256, precision=binding.PREC_BF16X3)
+            workloads.grow_middle_bond(c, 16, 8, 8, 256, 7, seed=n)
+            c.set_tune(tc_min=1)  # their own lists need no images, the batch's (its own launch shape) do
+            c.hpsi_flops()
+            out.append(c)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return out, torch.cuda.mem_get_info()[0]
+
+    def images_of_a_batch(ctxs, free):
+        batch = binding.Batch(ctxs)
+        x = workloads.gaussian(batch.offsets[-1], seed=1)
+        y = batch.hpsi(x)
+        batch.close()  # what stays are the members' images
+        return free - torch.cuda.mem_get_info()[0], y
+
+    ctxs, free = members()
+    images, ref = images_of_a_batch(ctxs, free)
+    for c in ctxs:
+        c.close()
+    assert images > 2**27
+    ctxs, free = members()
+    left = int(2.5 * images)
+    filler = torch.empty(free - left, dtype=torch.uint8, device="cuda")
+    taken, y = images_of_a_batch(ctxs, torch.cuda.mem_get_info()[0])
+    del filler
+    torch.cuda.empty_cache()
+    for c in ctxs:
+        c.close()
+    assert taken <= left / 3
+    assert np.max(np.abs(y - ref)) <= 1e-12 * np.max(np.abs(ref))
