@@ -4,17 +4,19 @@
 // SM and clock (measured; FP64 mma.sync 1.75), the integer pipe 63 32 x 32 + 64 bit
 // ones (mad.wide.s32, measured).  So a tile of doubles is read as a block-scaled
 // integer matrix: x = v 2^(E - 1079) with E the largest biased exponent of the tile
-// and v a rounded 58-bit integer, kept as two signed limbs v = hi 2^29 + lo, |hi|, |lo| <= 2^28.
+// and v a rounded integer, |v| < 2^57, kept as two signed limbs v = hi 2^29 + lo, |hi|, |lo| <= 2^28.
 // A dot product accumulates sum hi hi' and sum (hi lo' + lo hi') exactly in two 64-bit
 // registers: three multiply-adds per element product, the lo lo' term (2^-58 of the largest
 // product at most, of either sign) dropped.  For a depth of 32 |sum hi hi'| <= 2^61 and
-// |sum cross| <= 2^62.  The intermediate T = X Y is normalised back to 58 bits under an
-// exponent of its own.  The sum over tasks is FP64, as f may be any double.  Every FP64
-// operation may round by 2^-53 of its result; measured against FP64 full CI the products are
-// no less exact than FP64 ones (relative 2-norm of the error at L=12/M=800: 1.1e-15 in FP64).
-// A tile with a NaN, an infinity or an element outside 2^+-256 is multiplied in FP64 instead
-// (slow paths of the kernels), so those values
-// propagate as in FP64 arithmetic.
+// |sum cross| <= 2^62.  The intermediate T = X Y is normalised back to 57 bits under an
+// exponent of its own.  The sum over tasks is FP64, as f may be any double.
+//
+// The error is relative to a tile's largest elements: n 2^-55 max|X| max|Y| for a sum of n products
+// (tests/test_gpu_products.py has the terms), where FP64 has n 2^-53 times the sum of |x| |y|.  An
+// element below 2^-5 of its tile's largest has fewer than 53 bits, one below 2^-58 is zero.
+//
+// A tile with a NaN, an infinity or a largest element outside 2^+-256 is multiplied in FP64
+// instead (slow paths of the kernels), so those values propagate as in FP64 arithmetic.
 //
 // FP32 elements: one FP32 multiply-add per element product.
 #pragma once
@@ -29,7 +31,7 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------- element types
 
-// FX: 58-bit block-scaled integers in two limbs (from FP64), 8 bytes.
+// FX: 57-bit block-scaled integers in two limbs (from FP64), 8 bytes.
 // else: FP32, 4 bytes.
 template <bool FX>
 struct Arith;
@@ -58,7 +60,7 @@ __device__ __forceinline__ int2 limbs(long long v) {
 }
 __device__ __forceinline__ long long join(int2 v) { return ((long long)v.x << 29) + v.y; }
 
-// the 58-bit integer of x under tile exponent E (E >= x's own exponent field)
+// the integer of x, |v| < 2^57, under tile exponent E (E >= x's own exponent field)
 __device__ __forceinline__ int2 to_limbs(double x, int E) {
   const int h = __double2hiint(x);
   const int ex = (h >> 20) & 0x7ff;
