@@ -1031,10 +1031,14 @@ struct DevChain {
   int nspans = 0;
   SideStreams side;  // for the kernels of several classes
   bool forked() const { return pipe && side.ev[2]; }
-  bool on_cores() const {
-    for (int n : nitems)
-      if (n > 0) return true;
-    return false;
+  // whether the list has CUDA-core chunks and prepared operands take all of them
+  bool takes_images() const {
+    bool any = false;
+    for (const PipeClass &c : classes) {
+      if (c.items > 0 && (c.n > kPipeMaxN || c.p > 65535)) return false;
+      any |= c.items > 0;
+    }
+    return any;
   }
 
   // Run the list's CUDA-core chunks on prepared operands: o over the list's own operators, sp
@@ -1043,7 +1047,7 @@ struct DevChain {
   void prepare(const OpSet *o, std::vector<PsiSpan> sp, cudaStream_t s) {
     pipe = false;
     ops = o;
-    if (on_cores() && o && o->ready && sp.size() < (size_t(1) << 24)) {
+    if (takes_images() && o && o->ready && sp.size() < (size_t(1) << 24)) {
       const GivesBack none(nullptr, 0);
       try {
         build_entries(o, sp, s);
@@ -1203,6 +1207,7 @@ struct DevChain {
     tc_counter.release();
     nall = ntc = nred = npts = 0;
     for (int &n : nitems) n = 0;
+    for (PipeClass &c : classes) c = PipeClass();
     ntc_shape[0] = ntc_shape[1] = ntc_shape[2] = 0;
     nent = red_total = scratch_n = 0;
   }
@@ -1713,8 +1718,9 @@ static void build_images(dmrg_ctx *c, bool f32) {
 // The FP64 list on images (also made when a mixed-precision run first needs it).
 static void prepare_fp64(dmrg_ctx *c) {
   HPlan &P = c->plan;
-  if (P.ops.tried && P.chain.ops == &P.ops) return;
-  build_images(c, false);
+  if (P.chain.ops == &P.ops) return;
+  if (P.chain.takes_images()) build_images(c, false);
+  else if (P.chain32.ops != &P.ops) P.ops.release();  // an earlier position's
   P.chain.prepare(&P.ops, psi_spans(P.psi), c->stream);
 }
 
@@ -1765,7 +1771,8 @@ static void build_hplan(dmrg_ctx *c) {
     double fl32 = 0.0;
     hpsi_chainlist(c, true, CL32, fl32);
     P.chain32.upload(CL32, c->stream, false, true, c->tune, true);
-    build_images(c, true);
+    if (P.chain32.takes_images()) build_images(c, true);
+    else P.ops32.release();
     P.chain32.prepare(&P.ops32, psi_spans(Y), c->stream);
     CK(cudaStreamSynchronize(c->stream));
   } else if (c->prec == DMRG_PREC_BF16X3) {
@@ -1775,7 +1782,7 @@ static void build_hplan(dmrg_ctx *c) {
     double flt = 0.0;
     hpsi_chainlist(c, false, CLt, flt);
     P.chain32.upload(CLt, c->stream, true, true, c->tune, false);
-    if (P.chain32.on_cores()) {
+    if (P.chain32.takes_images()) {
       build_images(c, false);
       P.chain32.prepare(&P.ops, psi_spans(Y), c->stream);
     }
@@ -3846,7 +3853,7 @@ extern "C" int dmrg_batch_create(int n, dmrg_ctx *const *ctxs, dmrg_batch **out)
   }
   b->psi.alloc((size_t)std::max<long long>(b->off.back(), 1));
   b->sigma.alloc((size_t)std::max<long long>(b->off.back(), 1));
-  if (b->chain.on_cores()) batch_images(b.get(), b->stream);
+  if (b->chain.takes_images()) batch_images(b.get(), b->stream);
   b->chain.prepare(&b->ops, b->spans, b->stream);
   CK(cudaStreamCreateWithFlags(&b->own, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming));
@@ -4042,7 +4049,7 @@ extern "C" int dmrg_autotune(dmrg_ctx *c, int reps, double *best_ms, double *par
     y.alloc((size_t)std::max<int64_t>(n, 1));
     CK(launch_fill_guess(x.p, n, 0x5eedull, c->stream));
     const bool f32 = c->prec == DMRG_PREC_FP32;
-    build_images(c, f32);
+    if (tc || (f32 ? P.chain32 : P.chain).takes_images()) build_images(c, f32);
     best = autotune_chain(CL, tc, c->prec == DMRG_PREC_FP32, x.p, y.p, n, c->stream, c->dstatus.p, reps, c->tune,
                           ms, f32 ? &P.ops32 : &P.ops, psi_spans(P.psi));
     CK(cudaStreamSynchronize(c->stream));
