@@ -454,9 +454,11 @@ int dmrg_batch_free(dmrg_batch *batch);
  * this many equal-work chunks), min_chunk (no chunk lighter than this many
  * FLOPs), tc_min (output blocks with a side >= tc_min and both sides <= 128
  * run on the tensor-core kernel in DMRG_PREC_BF16X3), by_work (1: chunks
- * launched heaviest first; 0: in output-block order), flat_wide (1: chunks of
- * many tasks, or too few of them to fill the GPU, are shared by several groups
- * of warps of a CTA; 0: one group of warps per chunk) and tc_tiny (the tensor-core kernel's shape: 1 = every
+ * launched heaviest first; 0: in output-block order; chunks that do not run on
+ * the tensor cores go by their number of tasks first), flat_wide (FP64 chunks of
+ * many tasks, or too few of them to fill the GPU, are 1: shared by several groups
+ * of warps of a CTA, 0: run by one; FP32 chunks keep one order of their sum and
+ * are never shared) and tc_tiny (the tensor-core kernel's shape: 1 = every
  * block with m <= 64 and q and every task's p <= 32 runs on the 32-column
  * shape, five CTAs per SM, in a launch of its own; 0 = that shape only when
  * every block fits it, else the 64- and 128-row shapes).  Defaults: 8192, 2e5,

@@ -380,7 +380,7 @@ struct ChainTune {
   int tc_min = 33;
   int by_work = 0;     // 1: launch groups heaviest first; 0: in output-block order (operand locality)
   int orient = 1;      // run each entry in its cheaper association (split task lists)
-  int flat_wide = 1;   // CUDA-core kernels: 1 = several groups of warps may share a chunk, 0 = one per chunk
+  int flat_wide = 1;   // FP64 chunks: 1 = several groups of warps may share one, 0 = one per chunk
   int tc_tiny = 0;     // tensor-core kernel shapes: 1 = every block that fits the 32-column
                        // shape runs on it (a launch of its own), 0 = only when all blocks fit
 };
@@ -3988,7 +3988,8 @@ static ChainTune autotune_chain(const ChainList &CL, bool tc, bool ops32, const 
   for (int flip = 0; flip < 2; ++flip) {
     ChainTune t = best;
     if (flip == 0) t.by_work = 1 - best.by_work;
-    else t.flat_wide = 1 - best.flat_wide;
+    else if (!ops32) t.flat_wide = 1 - best.flat_wide;
+    else break;  // FP32 chunks keep one order of their sum and are never shared: nothing to choose
     const double ms = run(t);
     if (ms < best_ms) {
       best_ms = ms;
