@@ -116,13 +116,7 @@ __device__ __forceinline__ void load_rows(const char *p, bool full, const char *
 // from it, which saves them a conversion; the sum begins with what it adds taken off.
 constexpr float kMagic = 12582912.f;
 constexpr unsigned long long kMagicBits = 0x4b400000ull;
-constexpr unsigned long long kMagicSum = (kMagicBits << 40) + (kMagicBits << 30);  
-
-// Powers of two as values the compiler does not know: a multiply-add is one instruction, the shift
-// and the 64-bit addition that it would make of it are four.
-struct Powers {
-  int p0, p8, p10, p20, p30;
-};
+constexpr unsigned long long kMagicSum = (kMagicBits << 40) + (kMagicBits << 30);
 
 template <bool HALF>
 __device__ __forceinline__ void sums(const uint32_t (&a)[6][4], const uint32_t (&b)[6][2], float (&g)[7][4]) {
@@ -142,7 +136,7 @@ __device__ __forceinline__ void sums(const uint32_t (&a)[6][4], const uint32_t (
 }
 
 // s = a b (16 rows, 8 columns) over a depth of 16, or 8 (half)
-__device__ __forceinline__ void multiply(const uint32_t (&a)[6][4], const uint32_t (&b)[6][2], bool half, const Powers &w,
+__device__ __forceinline__ void multiply(const uint32_t (&a)[6][4], const uint32_t (&b)[6][2], bool half,
                                          long long (&s)[4]) {
   float g[7][4];
   if (half) sums<true>(a, b, g);
@@ -151,12 +145,12 @@ __device__ __forceinline__ void multiply(const uint32_t (&a)[6][4], const uint32
   for (int e = 0; e < 4; ++e) {
     s[e] = (long long)(0ull - kMagicSum);
     // units of 2^60: G_0 2^40 + G_1 2^30 + G_2 2^20 + G_3 2^10 + (G_4 + G_5 2^-10 + G_6 2^-20)
-    mad(s[e], __float2int_rn(fmaf(fmaf(g[6][e], 0x1p-10f, g[5][e]), 0x1p-10f, g[4][e])), w.p0);
-    mad(s[e], __float2int_rn(g[3][e]), w.p10);
-    mad(s[e], __float2int_rn(g[2][e]), w.p20);
-    mad(s[e], __float_as_int(g[1][e]), w.p30);
-    const int hi = (int)(s[e] >> 32) + __float_as_int(g[0][e]) * w.p8;
-    s[e] = (long long)((unsigned long long)(unsigned)hi << 32 | (unsigned)s[e]);
+    s[e] += __float2int_rn(fmaf(fmaf(g[6][e], 0x1p-10f, g[5][e]), 0x1p-10f, g[4][e]));
+    s[e] += (long long)__float2int_rn(g[3][e]) << 10;
+    s[e] += (long long)__float2int_rn(g[2][e]) << 20;
+    s[e] += (long long)__float_as_int(g[1][e]) << 30;
+    const unsigned hi = (unsigned)(s[e] >> 32) + (__float_as_uint(g[0][e]) << 8);
+    s[e] = (long long)((unsigned long long)hi << 32 | (unsigned)s[e]);
   }
 }
 
@@ -246,7 +240,7 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, SMW / (WC == 1 ? 4 : 
                      const int *__restrict__ nstacks, const ChainEntry *__restrict__ tasks,
                      const ChainGroup *__restrict__ G, const ChainItem *__restrict__ items,
                      const char *__restrict__ psi, const int *__restrict__ pexp, const double *__restrict__ psi64,
-                     uint64_t db, Powers w) {
+                     uint64_t db) {
   extern __shared__ __align__(16) unsigned char mma_smem[];
   __shared__ int te[2][WC][2];  // WC > 1: shifts of the chunks of T
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -337,7 +331,7 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, SMW / (WC == 1 ? 4 : 
             uint32_t b[6][2];
             load_block(Yk + j * kDigBlock, lane, b);
             long long s[4];
-            multiply(a, b, half, w, s);
+            multiply(a, b, half, s);
 #pragma unroll
             for (int u = 0; u < 2; ++u)
               if (u == j) {
@@ -404,10 +398,10 @@ __global__ void __launch_bounds__(WC == 1 ? 128 : 32 * WC, SMW / (WC == 1 ? 4 : 
           uint32_t a[6][4];
           load_rows(Z0 + off, have, Z0, false, lane, a);
           long long s[2][4];
-          multiply(a, td[0], half, w, s[0]);
+          multiply(a, td[0], half, s[0]);
           if (x1) {
             if (two) load_rows(Z1 + off, have, Z1, false, lane, a);
-            multiply(a, td[1], half, w, s[1]);
+            multiply(a, td[1], half, s[1]);
           }
 #pragma unroll
           for (int u = 0; u < NQ; ++u)
@@ -484,8 +478,7 @@ cudaError_t launch_mma(const PipeArgs &a, const ChainItem *items, const PipeClas
   auto kern = chain_mma_kernel<NQ, WC, SMW>;
   add_kernel_launches(1);
   kern<<<dim3(c.items, slices), 32 * warps, bytes, s>>>(a.e, a.stacks, a.nstacks, a.tasks, a.g, items,
-                                                        static_cast<const char *>(a.psi), a.pexp, a.psi64, a.db,
-                                                        Powers{1, 1 << 8, 1 << 10, 1 << 20, 1 << 30});
+                                                        static_cast<const char *>(a.psi), a.pexp, a.psi64, a.db);
   return cudaGetLastError();
 }
 
