@@ -71,6 +71,8 @@ TRAFFIC_PER_LAUNCH = {
     # chain_tc2 launches of one H.psi (one shape at M=3000, two at M=6000)
     ("c5a", 2, 3000, (8192.0, 200000.0, 1, 1, 1, 0)): 434.8e9 + 0.175e9,
     ("c5b", 2, 6000, (8192.0, 200000.0, 1, 1, 1, 0)): 1282.5e9 + 0.536e9,
+    # FP64 H.psi, every kernel of one call (chain_mma, psi images, reduction)
+    ("c2", 0, 512, (8192.0, 200000.0, 33, 0, 1, 0)): 11.45e9 + 0.37e9,
 }
 # Algorithmic bytes of one split-BF16x3 H.psi: the distinct pre-split operator tiles
 # (4 bytes per padded element, each read once), the psi tiles, psi and sigma
@@ -930,7 +932,7 @@ def fp64_step_line(args, wl, rank, world):
     if not args.no_mixed:
         for key, lp, what in (
                 ("mixed_fp32", 1, "FP32 operator copies for the Davidson matvecs"),
-                ("mixed_bf16x3", 2, "split-BF16x3 tensor-core matvecs (FP32 SIMT below the routing threshold)")):
+                ("mixed_bf16x3", 2, "split-BF16x3 tensor-core matvecs (FP64 below the routing threshold)")):
             m = run_gpu(args, wl, rank, world, lp, e2e=False, sample_clocks=False)
             ms = m["stats"]
             line[key] = {

@@ -576,12 +576,12 @@ int dmrg_debug_tasks(int L, int N, int two_sz, const double *h, const double *v,
  * the tensor-core kernel as DMRG_PREC_BF16X3 does; tune: NULL (defaults) or 5
  * doubles target_chunks, min_chunk, tc_min, by_work, tc_tiny as in
  * dmrg_set_tune.
- * counts (8): execution entries, chunks of the 32 x 32 tile kernel, of the
- * flattened-lane kernel, of the tensor-core kernel, reduction groups, tiles,
- * scratch elements, reduced elements.  Optional arrays (NULL to skip; sizes
+ * counts (8): execution entries, chunks of blocks above 32 x 32, of blocks up to
+ * 32 x 32, of the tensor-core kernel, reduction groups, 32 x 32 tiles of the
+ * blocks above that, scratch elements, reduced elements.  Optional arrays (NULL to skip; sizes
  * from counts): xs_out 8 per entry (psi offset of Y, n, p, Y row stride, Y
  * column stride, identity flags, X offset, Z offset; -1 for identity),
- * grp_out 8 per chunk (kernel 0/1/2, slot offset, slot row stride, slot column
+ * grp_out 8 per chunk (kind 0/1/2 in that order, slot offset, slot row stride, slot column
  * stride, m, q, first entry, entry count), red_out 8 per output block (first
  * reduced element, first slot offset, sigma offset, row stride, column stride,
  * m, q, chunk count).  Operator offsets are relative to each arena.

@@ -1,8 +1,8 @@
 // Element types and inner products of the triple products on the CUDA cores (sm_103a).
 //
 // FP64 products in fixed point.  The FP64 pipe of this GPU issues 2 multiply-adds per
-// SM and clock (measured; FP64 mma.sync 1.75), the integer pipe 63 32 x 32 + 64 bit
-// ones (mad.wide.s32, measured).  So a tile of doubles is read as a block-scaled
+// SM and clock (measured; FP64 mma.sync 1.75), the integer pipe 32 32 x 32 + 64 bit
+// ones (a multiply and an addition; measured, see mad()).  So a tile of doubles is read as a block-scaled
 // integer matrix: x = v 2^(E - 1079) with E the largest biased exponent of the tile
 // and v a rounded integer, |v| < 2^57, kept as two signed limbs v = hi 2^29 + lo, |hi|, |lo| <= 2^28.
 // A dot product accumulates sum hi hi' and sum (hi lo' + lo hi') exactly in two 64-bit
@@ -108,7 +108,9 @@ template <int S>
 __device__ __forceinline__ long long fold(long long hh, long long cr) {
   return (hh << S) + ((cr + (1ll << (28 - S))) >> (29 - S));
 }
-// One multiply-add instruction; mad.wide.s32 is compiled to a multiply and a 64-bit add.
+// d += a b.  A loop of nothing but mad.wide.s32 on the same operands measured 63 per SM and clock,
+// this form 32; but with mad.wide.s32 here the general kernel was slower (14 orbitals, M 1200 and
+// 300: 42.2 against 37.0 ms; M 1600 and 500: 85.9 against 73.7 ms).
 __device__ __forceinline__ void mad(long long &d, int a, int b) {
   asm("{\n\t.reg .s64 q;\n\tmul.wide.s32 q, %1, %2;\n\tadd.s64 %0, %0, q;\n\t}" : "+l"(d) : "r"(a), "r"(b));
 }
@@ -226,6 +228,5 @@ __device__ __forceinline__ double scaled(double f, int e) {
 __device__ __forceinline__ double muladd(double s, int2 v, double d) {
   return fma(s, (double)join(v), d);
 }
-__device__ __forceinline__ float muladd(float s, float v, float d) { return fmaf(s, v, d); }
 
 }  // namespace dmrg

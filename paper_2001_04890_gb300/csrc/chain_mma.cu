@@ -1,8 +1,8 @@
 // FP64 triple products of H.psi on the FP16 tensor pipe (sm_103a): D = sum_e f_e X_e Y_e Z_e
 // over prepared operands (Sec. 2.2.1, Eq. dgemm).
 //
-// The FP64 pipe issues 2 multiply-adds per SM and clock, the integer pipe 10 products of 58-bit
-// integers in two limbs (30 multiply-adds of 32 x 32 + 64 bits), the FP16 tensor pipe 1011
+// The FP64 pipe issues 2 multiply-adds per SM and clock, the integer pipe 10 products of 57-bit
+// integers in two limbs (32 multiply-adds of 32 x 32 + 64 bits), the FP16 tensor pipe 1011
 // products (mma.sync, all measured): at 26 per product of 58 bits, 39.  tcgen05 has 64 rows at
 // least and no FP64 or wide integer form; the blocks here have 1 to 120, most below 32, and the
 // 16 x 8 tile of mma.sync wastes less of them than its rate loses.
@@ -38,12 +38,12 @@
 // 8.2 ms, 12, M 800: 18.0 against 15.9 ms at equal occupancy), though D is then added to twice as
 // often.
 //
-// What bounds it: latency.  225 instructions a multiply of 26 (sums to integers, digits of T, D)
-// keep the tensor pipe 24 to 32% busy at the 4 warps a scheduler that registers allow.  Blocks are padded
+// What bounds it: latency.  206 to 310 instructions a multiply of 26 (sums to integers, digits of T, D)
+// keep the tensor pipe 24 to 33% busy at the 3 to 4 warps a scheduler that registers allow.  Blocks are padded
 // to 16 x 8 x 8: a third of the products at 24 orbitals, M 512, are of the problem.
 //
-// Time per H psi, limbs on the integer pipe -> this: 8 orbitals, M 64: 196 -> 179 us; 11, M 150:
-// 585 -> 357 us; 24, M 512: 11.2 -> 7.6 ms; 12, M 800: 23.1 -> 15.2 ms.
+// Time per H psi, limbs on the integer pipe -> this: 8 orbitals, M 64: 196 -> 178 us; 11, M 150:
+// 585 -> 353 us; 24, M 512: 11.2 -> 7.6 ms; 12, M 800: 23.1 -> 14.9 ms.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -465,9 +465,9 @@ int warps_per_slice(int n, int64_t tasks, int resident) {
 }
 
 // SMW: warps that an SM holds, registers against latency.  At 12 a warp has the 168 registers
-// that its sums, fragments and addresses want; at 16 it spills some outside the products, which
-// pays where there are warps enough.  12 / 16 for more than 32 columns: 12 orbitals, M 800: 16.3 /
-// 15.2 ms; for 32: 24 orbitals, M 512: 8.2 / 7.7 ms.
+// that its sums, fragments and addresses want; at 16 it spills some (340 to 380 bytes), which pays
+// where there are warps enough.  12 / 16 for every class but 0: 12 orbitals, M 800: 15.7 / 14.9 ms;
+// 24, M 512: 7.9 / 7.6 ms; with few chunks (11, M 150) it costs 340 / 353 us.
 template <int NQ, int WC, int SMW>
 cudaError_t launch_mma(const PipeArgs &a, const ChainItem *items, const PipeClass &c, int slices, bool share,
                        cudaStream_t s) {
@@ -498,8 +498,8 @@ cudaError_t launch_chain_mma(const PipeArgs &a, const ChainItem *items, const Pi
   if ((err = launch_mma<2, 2, 16>(a, i3, c[3], 2, false, s1)) != cudaSuccess) return err;
   if ((err = launch_mma<2, 1, 16>(a, i2, c[2], 2, wide != 0, s)) != cudaSuccess) return err;
   if ((err = launch_mma<2, 1, 16>(a, i1, c[1], 1, wide != 0, s1)) != cudaSuccess) return err;
-  // 12 / 16: 8 orbitals, M 64 (459 items): 181 / 196 us; 16 vectors, 24 orbitals, M 512 (14,368):
-  // 11.9 / 10.8 ms.  An item has four warps at most: the line is two waves of 16 an SM.
+  // 12 / 16: 8 orbitals, M 64 (459 items): 178 / 191 us; 24, M 512 (1,103): 7.56 / 7.43 ms; the batch of 16
+  // problems (14,368): 11.8 / 10.8 ms.  An item has four warps at most: the line is two waves of 16 an SM.
   if (c[0].items > 2 * 4 * 152) return launch_mma<1, 1, 16>(a, i0, c[0], 1, wide != 0, s2);
   return launch_mma<1, 1, 12>(a, i0, c[0], 1, wide != 0, s2);
 }

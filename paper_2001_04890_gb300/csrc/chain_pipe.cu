@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(256) pipe_entries_kernel(const ChainEntry *__r
         if (FX && (ef > 1023 + 100 || ef < 1023 - 100)) ex = -1;  // a coefficient that needs FP64
         p.w = FX ? (ex < 0 || ez < 0 ? INT_MIN : ex + ez + ef) : 0;
         p.src = g.first + b0 + (int)(unsigned)key[i];
-        const int cap = pipe_stack_cap(FX, g.tile0, g.m, g.q, e.n, e.p);
+        const int cap = pipe_stack_cap(FX, g.cls, g.m, g.q, e.n, e.p);
         head = (i - run0[i]) % cap == 0;
         st.e = g.first + b0 + i;
         st.ns = min(cap, run1[i] - i + 1);

@@ -314,7 +314,6 @@ struct ChainList {
   std::vector<Keyed> parts;     // further entries, built after ent, in part order
   std::vector<ChainGroup> grp;  // one per key, filled by finish()
   std::vector<ChainEntry, NoInitAlloc<ChainEntry>> flat;
-  int ntiles = 0;
   double flops = 0.0;
   size_t size() const {
     size_t n = ent.size();
@@ -354,15 +353,12 @@ struct ChainList {
     Keyed().swap(ent);  // the grouped copy is all that is used
     std::vector<Keyed>().swap(parts);
     grp.clear();
-    ntiles = 0;
     for (size_t k = 0; k < ng; ++k) {
       const int64_t c = start[k + 1] - start[k];
       if (c == 0) continue;
       ChainGroup g = protos[k];
       g.first = (int)start[k];
       g.count = (int)c;
-      g.tile0 = ntiles;
-      ntiles += ((g.m + 31) / 32) * ((g.q + 31) / 32);
       grp.push_back(g);
     }
   }
@@ -386,8 +382,8 @@ struct ChainTune {
 };
 // Host half of a task list's upload: the execution list (entries in their
 // cheaper association, cut into equal-work chunks when split_tasks), the launch
-// groups of the chunk kernels (CUDA cores: blocks above and up to 32 x 32; tensor
-// cores) and the ordered reduction of the chunk slots.
+// groups of the chunk kernels (not on the tensor cores: blocks above and up to 32 x 32;
+// on them) and the ordered reduction of the chunk slots.
 struct ExecPlan {
   std::vector<ChainEntry, NoInitAlloc<ChainEntry>> xs;
   std::vector<double, NoInitAlloc<double>> w;
@@ -443,7 +439,6 @@ static void plan_exec(const ChainList &CL, bool tensor_cores, bool split_tasks, 
     } else if (t.m <= 32 && t.q <= 32) {
       vf.push_back(t);
     } else {
-      t.tile0 = tiles;
       tiles += ((t.m + 31) / 32) * ((t.q + 31) / 32);
       vb.push_back(t);
     }
@@ -989,17 +984,18 @@ struct SideStreams {
 
 // A task list on the device.  When the tensor cores are enabled, output blocks
 // with both sides <= 128, one side >= tc_min and every entry's n, p <= 128 go
-// to the tensor-core kernel; of the rest, blocks of at most 32 x 32 go to the
-// flattened-lane warp kernel and larger ones to the 32 x 32 tile kernel.  With
-// split_tasks, every output block's entry list is cut into
-// chunks of about equal work; each chunk accumulates into its own slot of a
+// to the tensor-core kernel; the rest are cut into work items of the six classes
+// of chain_item_class, which run on prepared operands (chain_mma.cu in FP64,
+// chain_pipe.cu in FP32) where there are any, else on the general kernels
+// (chain_kernels.cu).  With split_tasks, every output block's entry list is cut into
+// chunks of about equal work; each chunk's sum goes to its own slot of a
 // scratch buffer and a reduction adds the slots in chunk order, so the result
 // does not depend on scheduling (bitwise repeatable) while the grid has
 // thousands of independent tasks.
 struct DevChain {
   DBuf<ChainEntry> ent, xent;
   DBuf<ChainGroup> all, cores;
-  DBuf<ChainItem> items;  // work items of the CUDA-core kernels, classes 4 to 0
+  DBuf<ChainItem> items;  // work items of the CUDA-core kernels, classes 5 to 0
   DBuf<ReduceGroup> red;
   DBuf<double> scratch;
   // tensor-core groups: entries with pre-split operand tiles (operators tiled
@@ -1126,7 +1122,7 @@ struct DevChain {
     for (PipeClass &c : classes) c = PipeClass();
     for (int i = 0; i < (int)vc.size(); ++i) {
       const int cls = chain_item_class(vc[i].m, vc[i].q, nmax[i], pmax[i]), cols = chain_item_cols(cls);
-      vc[i].tile0 = cls;
+      vc[i].cls = cls;
       for (int r0 = 0; r0 < vc[i].m; r0 += 32)
         for (int c0 = 0; c0 < vc[i].q; c0 += cols) {
           vi[cls].push_back({i, r0, c0, 0});
@@ -1618,15 +1614,12 @@ static void expand_hpsi_grouped(const std::vector<RPiece> &rps, const Arenas &A,
   for (size_t c = 0; c < nr; ++c) flops += fl[c];
   const std::vector<ChainGroup> protos = psi_protos(Y);
   CL.grp.clear();
-  CL.ntiles = 0;
   for (size_t g = 0; g < ng; ++g) {
     const int64_t n = start[g + 1] - start[g];
     if (n == 0) continue;
     ChainGroup G = protos[g];
     G.first = (int)start[g];
     G.count = (int)n;
-    G.tile0 = CL.ntiles;
-    CL.ntiles += ((G.m + 31) / 32) * ((G.q + 31) / 32);
     CL.grp.push_back(G);
   }
 }

@@ -102,7 +102,7 @@ int64_t pipe_image_size(bool f32, int rows, int cols);  // elements of one image
 cudaError_t launch_op_images(const OpSlab *s, int nslabs, int64_t nblocks, int16_t *exps, bool f32, cudaStream_t st);
 cudaError_t launch_psi_images(const PsiSpan *b, int nblocks, const double *psi, void *out, int *exps, bool f32,
                               cudaStream_t st);
-// The tasks of every group (tile0: its kernel class) as PipeEntry and their stacks (from the
+// The tasks of every group as PipeEntry and their stacks (from the
 // group's first entry on; nstacks per group); digits: sorted by psi block within the group.  *bad is
 // set if a task has a form that the kernels do not take.
 cudaError_t launch_pipe_entries(const ChainEntry *e, const ChainGroup *g, int ngroups, PipeEntry *out,

@@ -301,7 +301,7 @@ struct ChainGroup {
   int drs, dcs;
   int m, q;
   int first, count;
-  int tile0;
+  int cls;  // class of its work items (chain_item_class)
 };
 
 // Launch-shape decisions of the task lists (pure host logic).
