@@ -118,6 +118,28 @@ def test_renormalization_gives_images_back():
     assert np.array_equal(out[0], out[1])
 
 
+def test_a_new_position_gives_the_old_images_back():
+    """Any one allocation of the next position's plan may fail while the old position's images are there."""
+    ctx = _context(binding.PREC_FP64)
+    x = workloads.gaussian(ctx.psi_layout()[1], seed=3)
+    lay = ctx.enlarged_layout(1)
+    rng = np.random.default_rng(5)
+    O = np.concatenate([workloads.orthonormal_columns(int(d), min(int(d), 6), rng).ravel() for _, _, d in lay])
+    ctx.close()
+    ref = None
+    for n in [0] + list(range(1, 40)):
+        c = _context(binding.PREC_FP64)
+        c.hpsi(x)
+        c.renormalize(1, O, [min(int(d), 6) for _, _, d in lay])
+        z = workloads.gaussian(c.psi_layout()[1], seed=4)
+        binding.debug_fail_alloc(n)
+        y = c.hpsi(z)
+        binding.debug_fail_alloc(0)
+        ref = y if ref is None else ref
+        assert np.max(np.abs(y - ref)) <= 1e-12 * np.max(np.abs(ref)), n
+        c.close()
+
+
 def test_a_batch_keeps_its_contexts_images():
     ctx = _context(binding.PREC_FP64)
     x = workloads.gaussian(ctx.psi_layout()[1], seed=3)
